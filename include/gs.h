@@ -136,7 +136,12 @@ int gs_init(gs_sim* sim);
 
 /* Advance n >= 0 steps (asynchronous on the object's stream).  Step t -> t+1
  * draws r(seed, t, cell).  The plan (gs_set_plan) chooses the kernel; all
- * kernels give bitwise-identical results.  FP64 fields in GS_ARITH_DS, _FX
+ * kernels give bitwise-identical results.  Under the default plan
+ * (GS_KERNEL_AUTO) grids of up to 256^3 cells in their own IEEE arithmetic
+ * run up to 4096 steps in one launch (a cooperative one when it holds more
+ * than one step; its grid barrier is bounded by gs_set_fault's timeout);
+ * gs_get_plan then reports the z-march or plain kernel that larger grids
+ * would run.  FP64 fields in GS_ARITH_DS, _FX
  * or _FXF (periodic grids) stay in that arithmetic's packed form between the
  * steps of one call and are FP64 again when it ends, so n steps in one call
  * and in several calls can differ at the level of the FP64 rounding
@@ -199,7 +204,8 @@ int gs_set_plan_full(gs_sim* sim, const gs_plan* plan);
 int gs_get_plan_full(gs_sim* sim, gs_plan* out);
 
 /* Autotuner: time every candidate plan valid for this grid — the plain
- * kernel; z-march tiles x z-chunks x ring depths; for FP32, temporal
+ * kernel; the many-steps launch of gs_step (reported, set and cached as
+ * GS_KERNEL_AUTO, when it applies); z-march tiles x z-chunks x ring depths; for FP32, temporal
  * blocking at depths 2-8 with several tiles — over `steps_per_trial` steps
  * each (rounded up to a multiple of 12, then to whole passes of the plan's
  * depth; CUDA events on the object's stream, after warm-up launches), keep the

@@ -161,6 +161,8 @@ CUresult encode_act_4d(CUtensorMap* map, const void* base, int C, int L, long lo
 
 using namespace gs;
 
+static constexpr int kCtlWords = 6;  // gs_sim::d_err
+
 
 static bool finite_params(double a, double b, double c, double d, double e, double f)
 {
@@ -170,6 +172,8 @@ static bool finite_params(double a, double b, double c, double d, double e, doub
 
 static int default_plan(gs_sim* s)
 {
+    s->auto_plan = true;
+    s->auto_named = false;
     if (zmarch_supported(s->dtype, s->L)) {
         ZPlan pl;
         const int V = s->dtype == GS_F32 ? 4 : 2;
@@ -188,6 +192,17 @@ static int default_plan(gs_sim* s)
     s->kernel = GS_KERNEL_NAIVE;
     return GS_OK;
 }
+
+static constexpr int kResidentSteps = 4096;
+
+// whether the default plan means the resident kernel (the injected fault is
+// one of the TMA producer)
+static bool auto_is_resident(const gs_sim* s)
+{
+    return s->fault == 0 && s->p.arith == GS_ARITH_IEEE && resident_supported(s->L);
+}
+
+static bool runs_resident(const gs_sim* s) { return s->auto_plan && auto_is_resident(s); }
 
 static int encode_maps(gs_sim* s)
 {
@@ -214,9 +229,8 @@ static int check_common(int L, double Du, double Dv, double F, double k, double 
 
 static int finish_create(gs_sim* s, gs_sim** out)
 {
-    // the device error word, a pad word and the z-march kernel's two ticket words
-    GS_CUDA_TRY(cudaMalloc(&s->d_err, 4 * sizeof(int)));
-    GS_CUDA_TRY(cudaMemsetAsync(s->d_err, 0, 4 * sizeof(int), s->stream));
+    GS_CUDA_TRY(cudaMalloc(&s->d_err, kCtlWords * sizeof(int)));
+    GS_CUDA_TRY(cudaMemsetAsync(s->d_err, 0, kCtlWords * sizeof(int), s->stream));
     int rc = default_plan(s);
     if (!rc) rc = encode_maps(s);
     if (!rc) rc = launch_init(s->dtype, s->L, s->buf[0][0], s->buf[0][1], s->stream);
@@ -317,7 +331,7 @@ int gs_init(gs_sim* s)
     if (!s) return fail(GS_EINVAL, "sim is NULL");
     s->cur = 0;
     s->t = 0;
-    GS_CUDA_TRY(cudaMemsetAsync(s->d_err, 0, 4 * sizeof(int), s->stream));  // error word and tickets
+    GS_CUDA_TRY(cudaMemsetAsync(s->d_err, 0, kCtlWords * sizeof(int), s->stream));  // error word and tickets
     int rc = launch_init(s->dtype, s->L, s->buf[0][0], s->buf[0][1], s->stream);
     if (!rc) s->launches += 1;
     return rc;
@@ -328,6 +342,23 @@ int gs_step(gs_sim* s, int64_t n)
     if (!s) return fail(GS_EINVAL, "sim is NULL");
     if (n < 0) return fail(GS_EINVAL, "n=%lld must be >= 0", (long long)n);
     int64_t i = 0;
+    if (runs_resident(s)) {
+        // launches of at most kResidentSteps steps, so that no kernel runs for long
+        for (; i < n;) {
+            const int m = (int)std::min<int64_t>(n - i, kResidentSteps);
+            const int in = s->cur, outs = 1 - s->cur;
+            void* const u[2] = {s->buf[in][0], s->buf[outs][0]};
+            void* const v[2] = {s->buf[in][1], s->buf[outs][1]};
+            int rc = launch_resident(s->dtype, s->L, u, v, m, s->p, s->boundary == GS_BOUNDARY_HELD, s->t,
+                                     (unsigned*)(s->d_err + 4), s->d_err, s->timeout_ns, s->stream);
+            if (rc) return rc;
+            s->launches += 1;
+            s->cur = (m & 1) ? outs : in;
+            s->t += m;
+            i += m;
+        }
+        return GS_OK;
+    }
     if (s->kernel == GS_KERNEL_TBLOCK) {
         const int D = s->tp.depth;
         for (; i + D <= n; i += D) {
@@ -465,6 +496,7 @@ static int apply_plan(gs_sim* s, int kernel, int tile_x, int tile_y, int tile_z,
         return rc ? rc : encode_maps(s);
     }
     if (kernel == GS_KERNEL_NAIVE) {
+        s->auto_plan = false;
         s->kernel = GS_KERNEL_NAIVE;
         s->maps_ok = false;
         return GS_OK;
@@ -489,6 +521,8 @@ static int apply_plan(gs_sim* s, int kernel, int tile_x, int tile_y, int tile_z,
             s->kernel = old_kernel;
             s->zp = old;
             encode_maps(s);
+        } else {
+            s->auto_plan = false;
         }
         return rc;
     }
@@ -514,6 +548,7 @@ static int apply_plan(gs_sim* s, int kernel, int tile_x, int tile_y, int tile_z,
                 return rc;
             }
         }
+        s->auto_plan = false;
         return GS_OK;
     }
     return fail(GS_EINVAL, "kernel=%d not available", kernel);
@@ -539,6 +574,11 @@ static gs_plan current_plan(gs_sim* s)
 {
     gs_plan p{};
     p.kernel = s->kernel;
+    if (s->auto_plan && s->auto_named) {
+        p.kernel = GS_KERNEL_AUTO;
+        p.depth = 1;
+        return p;
+    }
     if (s->kernel == GS_KERNEL_ZMARCH) {
         p.tile_x = s->zp.tx; p.tile_y = s->zp.ty; p.tile_z = s->zp.tz; p.depth = 1; p.stages = s->zp.stages;
     } else if (s->kernel == GS_KERNEL_TBLOCK) {
@@ -558,6 +598,8 @@ int gs_autotune(gs_sim* s, int steps_per_trial, gs_plan* results, int max_result
     // candidate plans
     std::vector<gs_plan> cand;
     cand.push_back(gs_plan{GS_KERNEL_NAIVE, 0, 0, 0, 1, 0, 0.0});
+    // the default plan where it is more than its z-march tile (also tried below)
+    if (auto_is_resident(s)) cand.push_back(gs_plan{GS_KERNEL_AUTO, 0, 0, 0, 1, 0, 0.0});
     const int zt[][2] = {{128, 8}, {256, 4}, {64, 16}, {128, 4}, {64, 8}, {256, 8}, {128, 16}, {32, 16}, {128, 10},
                          {128, 12}, {256, 6}};
     for (auto& t : zt)
@@ -574,6 +616,7 @@ int gs_autotune(gs_sim* s, int steps_per_trial, gs_plan* results, int max_result
     // save the state
     const size_t bytes = (size_t)s->L * s->L * s->L * elem_size(s->dtype);
     const gs_plan saved_plan = current_plan(s);
+    const bool saved_auto = s->auto_plan, saved_named = s->auto_named;
     const int64_t t0 = s->t;
     const int cur0 = s->cur;
     void* bu = nullptr;
@@ -596,6 +639,7 @@ int gs_autotune(gs_sim* s, int steps_per_trial, gs_plan* results, int max_result
     for (size_t i = 0; i < cand.size() && !rc; ++i) {
         gs_plan& c = cand[i];
         if (apply_plan(s, c.kernel, c.tile_x, c.tile_y, c.tile_z, c.depth, c.stages) != GS_OK) continue;
+        s->auto_named = c.kernel == GS_KERNEL_AUTO;
         c = current_plan(s);
         // a whole number of passes of this plan's depth
         const int nc = c.kernel == GS_KERNEL_TBLOCK ? (n + c.depth - 1) / c.depth * c.depth : n;
@@ -626,8 +670,11 @@ int gs_autotune(gs_sim* s, int steps_per_trial, gs_plan* results, int max_result
     }
     s->cur = cur0;
     s->t = t0;
-    const gs_plan keep = (!rc && win.us_per_step >= 0) ? win : saved_plan;
-    int rc2 = apply_plan(s, keep.kernel, keep.tile_x, keep.tile_y, keep.tile_z, keep.depth, keep.stages);
+    const bool won = !rc && win.us_per_step >= 0;
+    const gs_plan keep = won ? win : saved_plan;
+    int rc2 = apply_plan(s, !won && saved_auto ? GS_KERNEL_AUTO : keep.kernel, keep.tile_x, keep.tile_y, keep.tile_z,
+                         keep.depth, keep.stages);
+    s->auto_named = won ? keep.kernel == GS_KERNEL_AUTO : saved_named;
     if (!rc && !rc2) s->plan_us = keep.us_per_step;
     if (bu) cudaFree(bu);
     if (bv) cudaFree(bv);
@@ -687,8 +734,10 @@ int gs_autotune_cached(gs_sim* s, int steps_per_trial, const char* path, gs_plan
     }
     if (have) {
         const gs_plan before = current_plan(s);
+        const bool before_auto = s->auto_plan, before_named = s->auto_named;
         if (apply_plan(s, found.kernel, found.tile_x, found.tile_y, found.tile_z, found.depth, found.stages) == GS_OK) {
             s->plan_us = found.us_per_step;
+            s->auto_named = found.kernel == GS_KERNEL_AUTO;
             if (best) {
                 *best = current_plan(s);
                 best->us_per_step = found.us_per_step;
@@ -697,7 +746,9 @@ int gs_autotune_cached(gs_sim* s, int steps_per_trial, const char* path, gs_plan
             return GS_OK;
         }
         // a plan this build or GPU no longer accepts: tune afresh
-        apply_plan(s, before.kernel, before.tile_x, before.tile_y, before.tile_z, before.depth, before.stages);
+        apply_plan(s, before_auto ? GS_KERNEL_AUTO : before.kernel, before.tile_x, before.tile_y, before.tile_z,
+                   before.depth, before.stages);
+        s->auto_named = before_named;
     }
     gs_plan b{};
     if ((rc = gs_autotune(s, steps_per_trial, nullptr, 0, nullptr, &b))) return rc;

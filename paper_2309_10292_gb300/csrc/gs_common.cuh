@@ -296,6 +296,11 @@ GS_D unsigned gs_atom_add_release_gpu(unsigned* p, unsigned v)
     return old;
 }
 
+GS_D void gs_red_add_release_gpu(unsigned* p, unsigned v)
+{
+    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
 GS_D unsigned gs_ld_acquire_gpu(const unsigned* p)
 {
     unsigned v;

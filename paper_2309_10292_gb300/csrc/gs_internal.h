@@ -92,6 +92,13 @@ int tblock_validate(int dtype, int L, const ZPlan& pl);
 int launch_tblock(int L, const ZPlan& pl, const void* u, const void* v, void* un, void* vn, const Params& p,
                   int64_t t, unsigned* tickets, cudaStream_t s);
 
+// Many steps of a small grid in one launch (gs_resident.cu): n steps from the
+// state in (u[0], v[0]), stepping between the two sets; the result is in set
+// n & 1.  bar: two zeroed words of device memory the launch leaves zeroed.
+bool resident_supported(int L);
+int launch_resident(int dtype, int L, void* const u[2], void* const v[2], int n, const Params& p, bool held, int64_t t,
+                    unsigned* bar, int* err, uint64_t timeout_ns, cudaStream_t s);
+
 }  // namespace gs
 
 // The single-grid simulation object (gs_api.cu owns its life cycle; the
@@ -108,8 +115,12 @@ struct gs_sim {
     int cur = 0;       // set holding the current state
     int64_t t = 0;     // step counter
     cudaStream_t stream = nullptr;
-    int* d_err = nullptr;  // 4 words: the error word, a pad word, the z-march kernel's two ticket words
+    // 6 words: the error word, a pad word, the z-march kernel's two ticket
+    // words, the resident kernel's two barrier words
+    int* d_err = nullptr;
     int kernel = GS_KERNEL_NAIVE;
+    bool auto_plan = false;   // the default plan: small grids run in the resident kernel
+    bool auto_named = false;  // ... chosen by the tuner, which reports it as GS_KERNEL_AUTO
     ZPlan zp{128, 8, 32, 4, 1};   // z-march plan (also runs the steps a blocked pass leaves over)
     ZPlan tp{64, 16, 64, 5, 2};   // temporal-blocking plan (kernel GS_KERNEL_TBLOCK)
     ZMaps maps[2];     // tensor maps reading set 0 / set 1

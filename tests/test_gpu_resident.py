@@ -1,0 +1,122 @@
+"""GPU tests of the many-steps launch that the default plan of a small grid takes.
+
+It must equal the one-thread-per-cell kernel bit for bit, whatever the edge
+(vector and scalar loads, one CTA to one per SM, runs of rows and bricks that
+do not divide the grid), the boundary and the grouping of steps into calls.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2309_10292_gb300 import gs
+from tests.gpu_util import PAPER, maxabs, need_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+def make(L, dtype, held=False, **kw):
+    need_cuda()
+    sim = gs.GrayScott(L, dtype=dtype, **dict(PAPER, **kw))
+    if held:
+        sim.boundary = gs.GS_BOUNDARY_HELD
+    return sim
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("noise,held", [(0.1, False), (0.0, False), (0.1, True), (0.0, True)])
+@pytest.mark.parametrize("L", [1, 2, 3, 4, 5, 12, 17, 32, 50, 63, 100])
+def test_small_grids_equal_the_plain_kernel(L, noise, held, dtype):
+    rng = np.random.default_rng(L)
+    u, v = rng.uniform(0, 1, (L, L, L)), rng.uniform(0, 0.5, (L, L, L))
+    sim, ref = (make(L, dtype, held, noise=noise, seed=2 ** 35 + 7) for _ in range(2))
+    ref.set_plan(gs.GS_KERNEL_NAIVE)
+    for s in (sim, ref):
+        s.write(u, v)
+        s.t = 5
+    for n in (1, 7, 0, 2):  # an odd and an even number of buffer swaps per call, one step without the barrier
+        sim.step(n)
+    ref.step(10)
+    assert sim.t == 15
+    for a, b in zip(sim.read(), ref.read()):
+        np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("L,dtype", [(180, "f32"), (184, "f32"), (256, "f32"), (255, "f32"), (256, "f64"), (145, "f64")])
+def test_largest_grids_equal_the_plain_kernel(L, dtype):
+    # both sides of the L2 footprint rule and the largest edge
+    sim, ref = (make(L, dtype, noise=0.1, seed=3) for _ in range(2))
+    ref.set_plan(gs.GS_KERNEL_NAIVE)
+    sim.step(5)
+    ref.step(5)
+    for a, b in zip(sim.read(), ref.read()):
+        np.testing.assert_array_equal(a, b)
+
+
+def test_more_steps_than_one_launch_holds():
+    L, n = 8, 4096 + 3
+    sim, ref = (make(L, "f32", noise=0.1, seed=3) for _ in range(2))
+    ref.set_plan(gs.GS_KERNEL_NAIVE)
+    before = gs.gs_launch_count(sim.handle)
+    sim.step(n)
+    assert gs.gs_launch_count(sim.handle) == before + 2
+    ref.step(n)
+    for a, b in zip(sim.read(), ref.read()):
+        np.testing.assert_array_equal(a, b)
+
+
+def test_captured_call_replays():
+    # a captured call advances from the state it was captured at, every time
+    import torch
+    L, n = 24, 6
+    st = torch.cuda.Stream()
+    sim = make(L, "f32", noise=0.1, seed=4, stream=st)
+    sim.step(2)
+    start = [t.clone() for t in sim.tensors()]
+    src = sim.tensors()
+    st.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=st):
+        sim.step(n)
+    got = []
+    for _ in range(2):
+        with torch.cuda.stream(st):
+            for a, b in zip(src, start):
+                a.copy_(b)
+            g.replay()
+        got.append(sim.read())
+    u0, v0 = oracle.init(L)
+    uo, vo = oracle.step(u0, v0, 2 + n, **dict(PAPER, noise=0.1, seed=4))
+    for (u, v) in got:
+        assert maxabs(u, uo) <= 1e-4 and maxabs(v, vo) <= 1e-4
+        np.testing.assert_array_equal(u, got[0][0])
+        np.testing.assert_array_equal(v, got[0][1])
+
+
+def test_grids_on_two_streams():
+    import torch
+    sims = [make(48, "f32", noise=0.1, seed=5 + i, stream=torch.cuda.Stream()) for i in range(2)]
+    for _ in range(20):
+        for s in sims:
+            s.step(9)
+    for i, s in enumerate(sims):
+        ref = make(48, "f32", noise=0.1, seed=5 + i)
+        ref.set_plan(gs.GS_KERNEL_NAIVE)
+        ref.step(180)
+        for a, b in zip(s.read(), ref.read()):
+            np.testing.assert_array_equal(a, b)
+
+
+def test_tuner_keeps_it_and_the_cache_remembers(tmp_path):
+    path = str(tmp_path / "plans.txt")
+    a = make(64, "f32", noise=0.1, seed=1)
+    best, hit = a.autotune_cached(path, steps_per_trial=48)
+    assert not hit and best["kernel"] == gs.GS_KERNEL_AUTO and a.plan == best
+    b = make(64, "f32", noise=0.1, seed=1)
+    best2, hit2 = b.autotune_cached(path, steps_per_trial=48)
+    assert hit2 and best2 == best and b.plan == best
+    before = gs.gs_launch_count(b.handle)
+    b.step(30)
+    assert gs.gs_launch_count(b.handle) == before + 1
+    b.set_plan(gs.GS_KERNEL_ZMARCH)
+    b.step(3)
+    assert gs.gs_launch_count(b.handle) == before + 4
