@@ -42,6 +42,7 @@
 
 #include "gs_common.cuh"
 #include "gs_internal.h"
+#include "gs_resident.cuh"
 #include "gs_tblock.cuh"
 
 namespace gs {
@@ -448,6 +449,91 @@ __global__ void __maxnreg__(sizeof(T) == 4 ? 76 : 96) gs_batch_kernel(const __gr
 }
 
 // ---------------------------------------------------------------------------
+// Small batches: every cell in L2, runs of rows instead of marched tiles.
+//
+// A z-marched item takes 0.9 us per plane whatever the bandwidth, so a step of
+// a batch that does not fill the chip with such items takes 28 us.  Here the
+// rows of all instances, in arena order, are cut into one equal share per CTA
+// (a few segments, each a run of rows of one instance); a group of cells is a
+// thread's turn with all its loads independent (gs_resident.cuh), and all CTAs
+// meet at a grid barrier between steps.
+// ---------------------------------------------------------------------------
+constexpr int kResSegs = 32;  // segments a CTA can hold
+// Arena size up to which it runs.  FP32: while the arena about fits L2 (us per
+// step, noise 0.1, this kernel against marched items: 64 of 32^3 (32 MB) 6.9 /
+// 27.8, 16 of 64^3 (64 MB) 10.9 / 27.8, 60 mixed (124 MB) 28.7 / 36.3, but 5 of
+// 128^3 (160 MB) 40.8 / 37.2).  FP64: bound by its pipe either way, this kernel
+// shares it out evenly (3 of 128^3, 192 MB: 276 / 388).
+static long long batch_res_bytes(int dtype) { return (dtype == GS_F32 ? 140ll : 256ll) << 20; }
+
+template <typename T>
+struct BResArgs {
+    T* arena;
+    const BInst* inst;
+    const int4* tab;  // [grid] (first segment, segments), then segments (instance, first row, rows)
+    BCtrl* ctrl;      // bar: barrier arrivals, next: CTAs done (both zero before the launch)
+    long long nsteps;
+    T Du6, Dv6, dt, noise24;
+    uint64_t timeout_ns;
+};
+
+template <typename T>
+struct BResSeg {
+    T* f[2][2];
+    ResRows r;
+    T F, Fk;
+    uint64_t seed;
+    GsKeys key[2];  // noise keys of the current and the next step
+};
+
+template <typename T, bool NOISE, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) gs_batch_res_kernel(const BResArgs<T> a)
+{
+    constexpr int V = GsVec<T>::N;
+    __shared__ BResSeg<T> seg[kResSegs];
+    const int tid = threadIdx.x;
+    const int4 head = a.tab[blockIdx.x];
+    const long long t0 = a.ctrl->t;
+    const int cur0 = a.ctrl->cur;
+    for (int j = tid; j < head.y; j += blockDim.x) {
+        const int4 d = a.tab[head.x + j];
+        const BInst& I = a.inst[d.x];
+        BResSeg<T>& g = seg[j];
+        for (int b = 0; b < 2; ++b)
+            for (int f = 0; f < 2; ++f) g.f[b][f] = a.arena + I.off[b][f];
+        g.r = ResRows{I.L, 0, I.L, d.y % I.L, d.y / I.L, d.z};
+        g.F = (T)I.F;
+        g.Fk = (T)I.Fk;
+        g.seed = (uint64_t)I.seed_hi << 32 | I.seed_lo;
+        if (NOISE) g.key[0] = gs_step_keys(g.seed, t0);
+    }
+    __syncthreads();
+    for (long long s = 0; s < a.nsteps; ++s) {
+        const int in = (cur0 + (int)(s & 1)) & 1;
+        for (int j = 0; j < head.y; ++j) {
+            const BResSeg<T>& g = seg[j];
+            const ResRows r = g.r;
+            const ResWalk<V> w(r, tid);
+            const GsCoef<T> c{a.Du6, a.Dv6, g.F, g.Fk, a.dt, a.noise24};
+            const GsKeys k = NOISE ? g.key[s & 1] : GsKeys{0, 0};
+            res_rows<T, V, NOISE, false>(r, w, g.f[in][0], g.f[in][1], g.f[in ^ 1][0], g.f[in ^ 1][1], c, k, tid);
+        }
+        if (s + 1 == a.nsteps) break;
+        if (NOISE)  // the slot was last read two steps ago
+            for (int j = tid; j < head.y; j += blockDim.x) seg[j].key[(s + 1) & 1] = gs_step_keys(seg[j].seed, t0 + s + 1);
+        if (res_grid_sync(&a.ctrl->bar, (unsigned)(s + 1) * gridDim.x, &a.ctrl->err, a.timeout_ns)) break;
+    }
+    // the last CTA to finish (every CTA has read t and cur) advances them
+    if (tid == 0) {
+        __threadfence();
+        if (atomicAdd(&a.ctrl->next, 1u) == gridDim.x - 1 && gs_ld_relaxed_gpu(&a.ctrl->err) == 0) {
+            a.ctrl->t = t0 + a.nsteps;
+            a.ctrl->cur = (cur0 + (int)(a.nsteps & 1)) & 1;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Temporally blocked batch (FP32, D = 2..4 steps per pass over HBM).
 //
 // The single-grid kernel's schedule (tb_item, gs_tblock.cuh) on the batch's
@@ -620,6 +706,11 @@ struct gs_batch {
     std::vector<int4> tb_base_items;
     int4* d_tb_items = nullptr;
     int tb_items_cap = 0, tb_nitems = 0, tb_items_grid = -1, tb_pe = 0, tb_grid = 0;
+    // small batches under the default plan run the L2-resident kernel
+    bool auto_plan = true;
+    int4* d_res_tab = nullptr;  // its table (built at its first capture)
+    std::vector<int4> h_res;    // ... and its contents (empty: it does not apply)
+    int res_grid = 0, res_segs = 0, res_groups = 0;
 };
 
 // The work item of z-chunk zc of a single-step table: (instance, c0, z0,
@@ -869,6 +960,89 @@ static cudaError_t capture_persistent(gs_batch* b, K kern, const A& args, int gr
     return cudaLaunchKernelEx(&cfg, kern, args);
 }
 
+// `launches` (into b->cap) as an executable graph, cooperative if possible
+template <typename Launches>
+static int capture_graph(gs_batch* b, cudaGraphExec_t* exec, Launches launches)
+{
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        cudaGraph_t g = nullptr;
+        GS_CUDA_TRY(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
+        const cudaError_t e2 = launches();
+        cudaError_t e3 = cudaStreamEndCapture(b->cap, &g);
+        cudaError_t e4 = cudaErrorUnknown;
+        if (e2 == cudaSuccess && e3 == cudaSuccess) e4 = cudaGraphInstantiate(exec, g, 0);
+        if (g) cudaGraphDestroy(g);
+        if (e2 == cudaSuccess && e3 == cudaSuccess && e4 == cudaSuccess) return GS_OK;
+        cudaGetLastError();
+        if (!b->cooperative) {
+            cudaError_t e = e2 != cudaSuccess ? e2 : (e3 != cudaSuccess ? e3 : e4);
+            return cuda_fail(e, "capturing the batched persistent launch");
+        }
+        b->cooperative = false;  // retry without the cooperative attribute (grids are sized to be co-resident)
+    }
+    return fail(GS_ECUDA, "capturing the batched persistent launch failed");
+}
+
+// The resident kernel's table: equal shares of the groups of all instances,
+// cut at rows.  False if some CTA would hold more segments than fit.
+static bool plan_res_table(gs_batch* b)
+{
+    const int V = b->dtype == GS_F32 ? 4 : 2;
+    long long total = 0;
+    for (int L : b->L) total += (long long)L * L * (L / V);
+    const int grid = (int)std::min<long long>(num_sms(), std::max<long long>(1, total / 128));
+    std::vector<int4> head(grid, int4{0, 0, 0, 0}), segs;
+    long long pos = 0;  // groups before the instance
+    int cta = 0;
+    auto limit = [&](int c) { return total * (c + 1) / grid; };
+    for (int i = 0; i < b->n; ++i) {
+        const int nxv = b->L[i] / V, rows = b->L[i] * b->L[i];
+        for (int r = 0; r < rows;) {
+            // rows up to the CTA's limit, at least one
+            while (cta + 1 < grid && pos + (long long)r * nxv >= limit(cta)) ++cta;
+            long long end = cta + 1 < grid ? (limit(cta) - pos + nxv - 1) / nxv : rows;
+            end = std::min<long long>(rows, std::max<long long>(end, r + 1));
+            if (head[cta].y == 0) head[cta].x = grid + (int)segs.size();
+            if (++head[cta].y > kResSegs) return false;
+            segs.push_back(make_int4(i, r, (int)end - r, 0));
+            r = (int)end;
+        }
+        pos += (long long)rows * nxv;
+    }
+    b->res_grid = grid;
+    b->res_segs = (int)segs.size();
+    b->res_groups = (int)((total + grid - 1) / grid);
+    head.insert(head.end(), segs.begin(), segs.end());
+    b->h_res = std::move(head);
+    return true;
+}
+
+// Whether the default plan means the L2-resident kernel (the injected faults
+// are those of the other kernels).
+static bool auto_is_resident(const gs_batch* b)
+{
+    return b->fault == 0 && !b->h_res.empty() && (long long)b->arena_bytes <= batch_res_bytes(b->dtype);
+}
+
+static bool runs_resident(const gs_batch* b) { return b->auto_plan && b->depth == 1 && auto_is_resident(b); }
+
+template <typename T, bool NOISE>
+static int res_capture(gs_batch* b, int64_t n, cudaGraphExec_t* exec)
+{
+    if (!b->d_res_tab) {
+        const size_t bytes = sizeof(int4) * b->h_res.size();
+        GS_CUDA_TRY(guarded_malloc((void**)&b->d_res_tab, bytes));
+        GS_CUDA_TRY(cudaMemcpy(b->d_res_tab, b->h_res.data(), bytes, cudaMemcpyHostToDevice));
+    }
+    const GsCoef<T> c = gs_make_coef<T>(b->Du, b->Dv, 0.0, 0.0, b->dt, b->noise);
+    const BResArgs<T> a{(T*)b->arena, b->d_inst, b->d_res_tab, b->d_ctrl, n, c.Du6, c.Dv6, c.dt, c.noise24, b->timeout_ns};
+    const bool wide = (long long)b->arena_bytes > kResL2Fit;  // as for a single grid
+    auto kern = wide ? gs_batch_res_kernel<T, NOISE, 1024> : gs_batch_res_kernel<T, NOISE, 512>;
+    const int maxt = wide ? 1024 : 512, turns = (b->res_groups + maxt - 1) / maxt;
+    const int threads = ((b->res_groups + turns - 1) / turns + 31) / 32 * 32;
+    return capture_graph(b, exec, [&] { return capture_persistent(b, kern, a, b->res_grid, threads, 0); });
+}
+
 // An n-step run as one graph: n / D blocked passes (D > 1), then the
 // remaining steps on the single-step kernel (which reads the step counter
 // and buffer set the blocked kernel leaves in the control block).
@@ -891,33 +1065,24 @@ static int batch_capture_t(gs_batch* b, int64_t n, cudaGraphExec_t* exec)
         const int rc = plain_prepare<T, NOISE>(b, rem, pa, psmem);
         if (rc) return rc;
     }
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        cudaGraph_t g = nullptr;
-        GS_CUDA_TRY(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e2 = cudaSuccess;
+    return capture_graph(b, exec, [&] {
+        cudaError_t e = cudaSuccess;
         if constexpr (D > 1) {
-            if (npasses) e2 = capture_persistent(b, gs_batch_tb_kernel<NOISE, D>, ta, b->tb_grid, kBtbThreads, tsmem);
+            if (npasses) e = capture_persistent(b, gs_batch_tb_kernel<NOISE, D>, ta, b->tb_grid, kBtbThreads, tsmem);
         }
-        if (e2 == cudaSuccess && rem)
-            e2 = capture_persistent(b, gs_batch_kernel<T, NOISE>, pa, b->grid, kBatchThreads, psmem);
-        cudaError_t e3 = cudaStreamEndCapture(b->cap, &g);
-        cudaError_t e4 = cudaErrorUnknown;
-        if (e2 == cudaSuccess && e3 == cudaSuccess) e4 = cudaGraphInstantiate(exec, g, 0);
-        if (g) cudaGraphDestroy(g);
-        if (e2 == cudaSuccess && e3 == cudaSuccess && e4 == cudaSuccess) return GS_OK;
-        cudaGetLastError();
-        if (!b->cooperative) {
-            cudaError_t e = e2 != cudaSuccess ? e2 : (e3 != cudaSuccess ? e3 : e4);
-            return cuda_fail(e, "capturing the batched persistent launch");
-        }
-        b->cooperative = false;  // retry without the cooperative attribute (grids are sized to be co-resident)
-    }
-    return fail(GS_ECUDA, "capturing the batched persistent launch failed");
+        if (e == cudaSuccess && rem)
+            e = capture_persistent(b, gs_batch_kernel<T, NOISE>, pa, b->grid, kBatchThreads, psmem);
+        return e;
+    });
 }
 
 static int batch_capture(gs_batch* b, int64_t n, cudaGraphExec_t* exec)
 {
     const bool noise = b->noise != 0.0;
+    if (runs_resident(b)) {
+        if (b->dtype != GS_F32) return noise ? res_capture<double, true>(b, n, exec) : res_capture<double, false>(b, n, exec);
+        return noise ? res_capture<float, true>(b, n, exec) : res_capture<float, false>(b, n, exec);
+    }
     if (b->dtype != GS_F32)
         return noise ? batch_capture_t<double, true, 1>(b, n, exec) : batch_capture_t<double, false, 1>(b, n, exec);
     switch (b->depth) {
@@ -956,6 +1121,7 @@ int gs_batch_destroy(gs_batch* b)
     guarded_free(b->d_ctrl);
     guarded_free(b->d_tb_rows);
     guarded_free(b->d_tb_items);
+    guarded_free(b->d_res_tab);
     if (b->cap) cudaStreamDestroy(b->cap);
     delete b;
     return GS_OK;
@@ -997,6 +1163,11 @@ int gs_batch_create(int n, const int* L, const double* F, const double* k, doubl
     const int a128 = 128 / esz;
     const int tile_cells = kBatchConsumers * V;
     int box_elems = 0;
+    // z-chunk: 32 planes, 16 where that leaves fewer than two items per CTA
+    // (64 grids of 64^3: 58 against 51 us a step; 100 of them: 76.0 against 75.7)
+    long long items32 = 0;
+    for (int i = 0; i < n; ++i) items32 += (long long)run_tiles(L[i], tile_cells) * ((L[i] + 31) / 32);
+    b->tz = items32 < 4ll * num_sms() ? 16 : 32;
     // instance table, arena offsets, work items
     int nit = 0;
     long long off = 0;
@@ -1075,6 +1246,7 @@ int gs_batch_create(int n, const int* L, const double* F, const double* k, doubl
             (e = cudaMemset(b->d_ctrl, 0, sizeof(BCtrl))) != cudaSuccess)
             rc = cuda_fail(e, "uploading the batch tables");
     }
+    plan_res_table(b);
     if (rc == GS_OK) rc = upload_items(b, b->base_items);
     if (rc == GS_OK) rc = gs_batch_init(b);
     if (rc != GS_OK) {
@@ -1169,6 +1341,7 @@ int gs_batch_autotune(gs_batch* b, int steps_per_trial, int* best_tile_z, int* b
     // whole passes at every depth: the trial length is a multiple of 12
     const int trial = (steps_per_trial + 11) / 12 * 12;
     const int tz0 = b->tz, st0 = b->stages, d0 = b->depth;
+    const bool auto0 = b->auto_plan;
     const int64_t t0 = b->t;
     const int cur0 = b->cur;
     void* saved = nullptr;
@@ -1182,6 +1355,31 @@ int gs_batch_autotune(gs_batch* b, int steps_per_trial, int* best_tile_z, int* b
         rc = cuda_fail(e, "batch autotune save");
     int win_tz = tz0, win_st = st0, win_d = d0;
     double win_us = -1.0;
+    bool win_auto = false;
+    auto time_plan = [&](double& us) -> int {
+        int r = gs_batch_step(b, trial);  // captures the graph, warms up
+        if (!r) r = gs_batch_sync(b);
+        if (!r && (e = cudaEventRecord(e0, b->stream)) != cudaSuccess) r = cuda_fail(e, "event");
+        if (!r) r = gs_batch_step(b, trial);
+        if (!r && (e = cudaEventRecord(e1, b->stream)) != cudaSuccess) r = cuda_fail(e, "event");
+        if (!r) r = gs_batch_sync(b);
+        float ms = 0.f;
+        if (!r && (e = cudaEventElapsedTime(&ms, e0, e1)) != cudaSuccess) r = cuda_fail(e, "event");
+        us = 1e3 * ms / trial;
+        return r;
+    };
+    if (!rc && auto_is_resident(b)) {
+        // the default plan where it is more than its z-chunk and ring (also tried below)
+        rc = gs_batch_set_depth(b, 1);
+        if (!rc) {
+            b->auto_plan = true;
+            rc = time_plan(win_us);
+        }
+        win_auto = !rc;
+        win_tz = 32;
+        win_st = 8;
+        win_d = 1;
+    }
     for (int depth = 1; depth <= kBtbMaxDepth && !rc; ++depth) {
         if (depth > 1 && b->dtype != GS_F32) break;
         for (int tz : {16, 32, 64, 128}) {
@@ -1191,24 +1389,14 @@ int gs_batch_autotune(gs_batch* b, int steps_per_trial, int* best_tile_z, int* b
                 if (depth > 1 && st != 4) continue;   // the blocked form has no TMA ring
                 if (gs_batch_set_plan(b, tz, st) != GS_OK) continue;  // a ring that does not fit
                 if (gs_batch_set_depth(b, depth) != GS_OK) continue;  // no blocked tile for some instance
-                int r = gs_batch_step(b, trial);                      // captures the graph, warms up
-                if (!r) r = gs_batch_sync(b);
-                if (!r && (e = cudaEventRecord(e0, b->stream)) != cudaSuccess) r = cuda_fail(e, "event");
-                if (!r) r = gs_batch_step(b, trial);
-                if (!r && (e = cudaEventRecord(e1, b->stream)) != cudaSuccess) r = cuda_fail(e, "event");
-                if (!r) r = gs_batch_sync(b);
-                float ms = 0.f;
-                if (!r && (e = cudaEventElapsedTime(&ms, e0, e1)) != cudaSuccess) r = cuda_fail(e, "event");
-                if (r) {
-                    rc = r;
-                    break;
-                }
-                const double us = 1e3 * ms / trial;
+                double us = 0.0;
+                if ((rc = time_plan(us))) break;
                 if (win_us < 0 || us < win_us) {
                     win_us = us;
                     win_tz = tz;
                     win_st = depth > 1 ? st0 : st;
                     win_d = depth;
+                    win_auto = false;
                 }
             }
         }
@@ -1226,6 +1414,10 @@ int gs_batch_autotune(gs_batch* b, int steps_per_trial, int* best_tile_z, int* b
     b->ctrl_dirty = true;
     int rc2 = rc ? gs_batch_set_plan(b, tz0, st0) : gs_batch_set_plan(b, win_tz, win_st);
     if (!rc2) rc2 = gs_batch_set_depth(b, rc ? d0 : win_d);
+    if (!rc2 && (rc ? auto0 : win_auto)) {
+        b->auto_plan = true;
+        drop_graphs(b);
+    }
     if (rc) return rc;
     if (rc2) return rc2;
     if (best_tile_z) *best_tile_z = win_tz;
@@ -1330,6 +1522,7 @@ int gs_batch_set_plan(gs_batch* b, int tile_z, int stages)
     GS_CUDA_TRY(cudaMemcpy(b->d_inst, b->h_inst.data(), sizeof(BInst) * b->n, cudaMemcpyHostToDevice));
     b->tz = tile_z;
     b->stages = stages;
+    b->auto_plan = false;
     drop_graphs(b);
     if (b->depth > 1) return build_tb_tables(b, b->depth);  // the blocked items follow the z-chunk
     return GS_OK;
@@ -1345,6 +1538,7 @@ int gs_batch_set_depth(gs_batch* b, int depth)
         if (rc) return rc;
     }
     b->depth = depth;
+    b->auto_plan = false;
     drop_graphs(b);
     return GS_OK;
 }
@@ -1355,7 +1549,8 @@ int gs_batch_guard_check(gs_batch* b, int64_t* bad)
     GS_CUDA_TRY(cudaStreamSynchronize(b->stream));
     int64_t n = 0;
     for (const void* p : {(const void*)b->arena, (const void*)b->d_inst, (const void*)b->d_items, (const void*)b->d_maps,
-                          (const void*)b->d_ctrl, (const void*)b->d_tb_rows, (const void*)b->d_tb_items}) {
+                          (const void*)b->d_ctrl, (const void*)b->d_tb_rows, (const void*)b->d_tb_items,
+                          (const void*)b->d_res_tab}) {
         const int64_t r = guarded_check(p);
         if (r < 0) return fail(GS_ECUDA, "reading a guard band failed");
         n += r;
@@ -1368,8 +1563,9 @@ int gs_batch_info(gs_batch* b, int* grid, int* items, int* cooperative, int64_t*
 {
     if (!b) return fail(GS_EINVAL, "batch is NULL");
     if (depth) *depth = b->depth;
-    if (grid) *grid = b->depth > 1 ? b->tb_grid : b->grid;
-    if (items) *items = b->depth > 1 ? b->tb_nitems : b->nitems;
+    const bool res = runs_resident(b) && b->d_res_tab;
+    if (grid) *grid = res ? b->res_grid : b->depth > 1 ? b->tb_grid : b->grid;
+    if (items) *items = res ? b->res_segs : b->depth > 1 ? b->tb_nitems : b->nitems;
     if (cooperative) *cooperative = b->cooperative ? 1 : 0;
     if (launches) *launches = b->launches;
     return GS_OK;

@@ -20,6 +20,7 @@
 
 #include "gs_common.cuh"
 #include "gs_internal.h"
+#include "gs_resident.cuh"
 
 namespace gs {
 
@@ -37,130 +38,34 @@ struct ResArgs {
     uint64_t timeout_ns;
 };
 
-// V cells of one 16-byte vector, or one cell (V = 1: edges L that are no
-// multiple of the vector)
-template <typename T, int V>
-GS_D void res_load(const T* p, T* r)
-{
-    if constexpr (V == 1) r[0] = *p;
-    else gs_unpack<T>(*reinterpret_cast<const typename GsVec<T>::type*>(p), r);
-}
-
-template <typename T, int V>
-GS_D void res_store(T* p, const T* r)
-{
-    if constexpr (V == 1) *p = r[0];
-    else *reinterpret_cast<typename GsVec<T>::type*>(p) = gs_pack<T>(r);
-}
-
 template <typename T, int V, bool NOISE, bool HELD, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) gs_resident_kernel(const ResArgs<T> a)
 {
-    const int L = a.L, nxv = L / V, LL = L * L;
-    const int tid = threadIdx.x;
+    const int L = a.L, tid = threadIdx.x;
     // this CTA's rows: a brick (a y range times a z range), or with ny = 0 a
-    // run of the rows in (y, z) order; either way rows ylo..yhi-1 of plane
-    // after plane from (ys, zs) on, nrow of them
-    int ylo = 0, yhi = L, ys, zs, nrow;
+    // run of the rows in memory order
+    ResRows r{L, 0, L, 0, 0, 0};
     if (a.ny) {
         const int by = blockIdx.x % a.ny, bz = blockIdx.x / a.ny;
-        ylo = L * by / a.ny;
-        yhi = L * (by + 1) / a.ny;
-        ys = ylo;
-        zs = L * bz / a.nz;
-        nrow = (yhi - ylo) * (L * (bz + 1) / a.nz - zs);
+        r.ylo = L * by / a.ny;
+        r.yhi = L * (by + 1) / a.ny;
+        r.ys = r.ylo;
+        r.zs = L * bz / a.nz;
+        r.nrow = (r.yhi - r.ylo) * (L * (bz + 1) / a.nz - r.zs);
     } else {
-        const int r0 = (int)((long long)LL * blockIdx.x / gridDim.x);
-        nrow = (int)((long long)LL * (blockIdx.x + 1) / gridDim.x) - r0;
-        zs = r0 / L;
-        ys = r0 - zs * L;
+        const long long LL = (long long)L * L;
+        const int r0 = (int)(LL * blockIdx.x / gridDim.x);
+        r.nrow = (int)(LL * (blockIdx.x + 1) / gridDim.x) - r0;
+        r.zs = r0 / L;
+        r.ys = r0 - r.zs * L;
     }
-    const int nr = yhi - ylo, ng = nrow * nxv;
-    // this thread's first group (x fastest, then y, then z) and the step to
-    // its next one as (x, y, z) increments
-    const int r0 = tid / nxv, xv0 = tid - r0 * nxv;
-    const int dr = blockDim.x / nxv, dxv = blockDim.x - dr * nxv;
-    const int q0 = ys - ylo + r0, dz = dr / nr, dy = dr - dz * nr;
-    const int z00 = zs + q0 / nr, y00 = ylo + q0 % nr;
-    bool stop = false;
-    for (int s = 0; s < a.n && !stop; ++s) {
+    const ResWalk<V> w(r, tid);
+    for (int s = 0; s < a.n; ++s) {
         const GsKeys k = NOISE ? gs_step_keys(a.seed, a.t + s) : GsKeys{0, 0};
-        const uint32_t kk2 = gs_kk2(k);
         const bool even = (s & 1) == 0;
-        // no __restrict__: another CTA writes what this one reads a step later
-        const T* u = even ? a.u0 : a.u1;
-        const T* v = even ? a.v0 : a.v1;
-        T* un = even ? a.u1 : a.u0;
-        T* vn = even ? a.v1 : a.v0;
-        int xv = xv0, y = y00, z = z00;
-        for (int g = tid; g < ng; g += blockDim.x) {
-            // 32-bit indices: L <= 256
-            const int x = xv * V, row = (z * L + y) * L, i = row + x;
-            const int iym = y == 0 ? i + LL - L : i - L;
-            const int iyp = y == L - 1 ? i - (LL - L) : i + L;
-            const int izm = z == 0 ? i + (L - 1) * LL : i - LL;
-            const int izp = z == L - 1 ? i - (L - 1) * LL : i + LL;
-            const int ixl = x == 0 ? row + L - 1 : i - 1;
-            const int ixr = x + V == L ? row : i + V;
-            T cu[V], cv[V], pu[V], pv[V], nu[V], nv[V], ymu[V], ypu[V], ymv[V], ypv[V], ou[V], ov[V];
-            res_load<T, V>(u + i, cu);
-            res_load<T, V>(u + iym, ymu);
-            res_load<T, V>(u + iyp, ypu);
-            res_load<T, V>(u + izm, pu);
-            res_load<T, V>(u + izp, nu);
-            res_load<T, V>(v + i, cv);
-            res_load<T, V>(v + iym, ymv);
-            res_load<T, V>(v + iyp, ypv);
-            res_load<T, V>(v + izm, pv);
-            res_load<T, V>(v + izp, nv);
-            const T xlu = u[ixl], xru = u[ixr], xlv = v[ixl], xrv = v[ixr];
-            if constexpr (V == 1) {
-                const T su = gs_nsum(xlu, xru, ymu[0], ypu[0], pu[0], nu[0]);
-                const T sv = gs_nsum(xlv, xrv, ymv[0], ypv[0], pv[0], nv[0]);
-                gs_update<T, NOISE>(a.c, cu[0], cv[0], su, sv, NOISE ? (T)gs_noise_num((uint32_t)i, k) : (T)0, ou[0],
-                                    ov[0]);
-            } else {
-                const uint32_t pre = NOISE ? gs_group_pre((uint32_t)i, k) : 0u;
-                gs_update_group<T, NOISE>(a.c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru, xlv, xrv,
-                                          ou, ov);
-            }
-            if (HELD) {
-                const bool face = y == 0 || y == L - 1 || z == 0 || z == L - 1;
-#pragma unroll
-                for (int e = 0; e < V; ++e)
-                    if (face || (e == 0 && x == 0) || (e == V - 1 && x + V == L)) {
-                        ou[e] = cu[e];
-                        ov[e] = cv[e];
-                    }
-            }
-            res_store<T, V>(un + i, ou);
-            res_store<T, V>(vn + i, ov);
-            xv += dxv;
-            y += dy;
-            z += dz;
-            if (xv >= nxv) { xv -= nxv; ++y; }
-            if (y >= yhi) { y -= nr; ++z; }
-        }
-        if (s + 1 == a.n) break;
-        // grid barrier: the CTA's stores are ordered before its arrival (the
-        // barrier makes them thread 0's predecessors), every other CTA's
-        // before thread 0's acquire, and that before this CTA's next loads
-        __syncthreads();
-        int bad = 0;
-        if (tid == 0) {
-            gs_red_add_release_gpu(a.bar, 1u);
-            const unsigned want = (unsigned)(s + 1) * gridDim.x;
-            if ((int)(gs_ld_acquire_gpu(a.bar) - want) < 0) {
-                const uint64_t t0 = gs_globaltimer();
-                while ((int)(gs_ld_acquire_gpu(a.bar) - want) < 0)
-                    if (gs_globaltimer() - t0 > a.timeout_ns) {
-                        gs_report(a.err, GS_DERR_TIMEOUT);
-                        bad = 1;
-                        break;
-                    }
-            }
-        }
-        stop = __syncthreads_or(bad);
+        res_rows<T, V, NOISE, HELD>(r, w, even ? a.u0 : a.u1, even ? a.v0 : a.v1, even ? a.u1 : a.u0,
+                                    even ? a.v1 : a.v0, a.c, k, tid);
+        if (s + 1 < a.n && res_grid_sync(a.bar, (unsigned)(s + 1) * gridDim.x, a.err, a.timeout_ns)) break;
     }
     // the last CTA to finish zeroes both words for the next launch
     if (a.n > 1 && tid == 0) {
@@ -171,9 +76,6 @@ __global__ void __launch_bounds__(MAXT, 1) gs_resident_kernel(const ResArgs<T> a
         }
     }
 }
-
-// Footprint (both buffer sets) up to which the loads are L2 hits throughout.
-static constexpr long long kL2Fit = 96ll << 20;
 
 template <typename T, int V, bool NOISE, bool HELD>
 static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, const Params& p, int64_t t,
@@ -218,7 +120,7 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
     // 512 threads of up to 128 registers while the fields fit L2; beyond that,
     // and with scalar loads, latency wants the 1024 (FP32 160^3: 10.4 against
     // 11.4 us; 192^3: 25.0 against 19.8 us; 101^3: 8.2 against 6.4 us)
-    const bool wide = V == 1 || 4 * (long long)sizeof(T) * L * rows_all > kL2Fit;
+    const bool wide = V == 1 || 4 * (long long)sizeof(T) * L * rows_all > kResL2Fit;
     const int maxt = wide ? 1024 : 512;
     const int ng = nxv * rows, turns = (ng + maxt - 1) / maxt;
     const int threads = ((ng + turns - 1) / turns + 31) / 32 * 32;

@@ -120,3 +120,59 @@ def test_tuner_keeps_it_and_the_cache_remembers(tmp_path):
     b.set_plan(gs.GS_KERNEL_ZMARCH)
     b.step(3)
     assert gs.gs_launch_count(b.handle) == before + 4
+
+
+# ---------------------------------------------------------------------------
+# Small batches (equal shares of all instances' rows per CTA)
+# ---------------------------------------------------------------------------
+def batch_pair(Ls, dtype, noise):
+    need_cuda()
+    F, k = np.linspace(0.02, 0.05, len(Ls)), np.linspace(0.05, 0.065, len(Ls))
+    return [gs.GrayScottBatch(Ls, F, k, noise=noise, seed=2 ** 33 + 1, dtype=dtype) for _ in range(2)]
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("Ls,noise", [([4], 0.1), ([4, 8, 12, 100], 0.1), ([64, 20, 36] * 5, 0.0), ([32] * 40, 0.1),
+                                      ([160, 4, 4], 0.1)])
+def test_small_batches_equal_marched_items(Ls, noise, dtype):
+    a, b = batch_pair(Ls, dtype, noise)
+    gs.gs_batch_set_plan(b.handle, 8, 4)
+    for n in (1, 6, 1, 3):
+        a.step(n)
+    assert a.info["grid"] <= 152 and a.t == 11
+    b.step(11)
+    for i in range(len(Ls)):
+        for x, y in zip(a.read(i), b.read(i)):
+            np.testing.assert_array_equal(x, y)
+    # per-instance launches and a new step index continue from its state
+    for x in (a, b):
+        x.step_sequential(2)
+        x.t = 40
+        x.step(5)
+    for x, y in zip(a.read(0), b.read(0)):
+        np.testing.assert_array_equal(x, y)
+
+
+def test_batch_of_many_tiny_grids_keeps_marched_items():
+    # more segments than a CTA of the row-sharing kernel holds
+    a, b = batch_pair([4] * 300 + [128], "f32", 0.1)
+    gs.gs_batch_set_plan(b.handle, 32, 8)
+    for x in (a, b):
+        x.step(4)
+    assert a.info["grid"] == b.info["grid"] > 152  # two CTAs per SM, as many items as there are
+    for i in (0, 150, 299, 300):
+        for x, y in zip(a.read(i), b.read(i)):
+            np.testing.assert_array_equal(x, y)
+
+
+def test_batch_tuner_keeps_row_shares():
+    a, b = batch_pair([32, 48, 64] * 4, "f32", 0.0)
+    plan = a.autotune(steps_per_trial=48)
+    assert (plan["tile_z"], plan["stages"], plan["depth"]) == (32, 8, 1)
+    assert a.info["grid"] == 152 and a.t == 0
+    a.step(9)
+    gs.gs_batch_set_plan(b.handle, 32, 8)
+    b.step(9)
+    for i in (0, 5, 11):
+        for x, y in zip(a.read(i), b.read(i)):
+            np.testing.assert_array_equal(x, y)
