@@ -137,8 +137,9 @@ int gs_init(gs_sim* sim);
 /* Advance n >= 0 steps (asynchronous on the object's stream).  Step t -> t+1
  * draws r(seed, t, cell).  The plan (gs_set_plan) chooses the kernel; all
  * kernels give bitwise-identical results.  Under the default plan
- * (GS_KERNEL_AUTO) grids of up to 256^3 cells in their own IEEE arithmetic
- * run up to 4096 steps in one launch (a cooperative one when it holds more
+ * (GS_KERNEL_AUTO) grids of up to 256^3 cells (160^3, or 180^3 with an odd
+ * edge, in GS_ARITH_DS, _FX or _FXF with the periodic boundary) run up to 4096
+ * steps in one launch (a cooperative one when it holds more
  * than one step; its grid barrier is bounded by gs_set_fault's timeout);
  * gs_get_plan then reports the z-march or plain kernel that larger grids
  * would run.  FP64 fields in GS_ARITH_DS, _FX

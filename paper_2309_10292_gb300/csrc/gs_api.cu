@@ -199,7 +199,8 @@ static constexpr int kResidentSteps = 4096;
 // one of the TMA producer)
 static bool auto_is_resident(const gs_sim* s)
 {
-    return s->fault == 0 && s->p.arith == GS_ARITH_IEEE && resident_supported(s->L);
+    if (s->fault != 0 || !resident_supported(s->L, s->p.arith)) return false;
+    return s->p.arith == GS_ARITH_IEEE || s->boundary == GS_BOUNDARY_PERIODIC;
 }
 
 static bool runs_resident(const gs_sim* s) { return s->auto_plan && auto_is_resident(s); }
@@ -349,7 +350,9 @@ int gs_step(gs_sim* s, int64_t n)
             const int in = s->cur, outs = 1 - s->cur;
             void* const u[2] = {s->buf[in][0], s->buf[outs][0]};
             void* const v[2] = {s->buf[in][1], s->buf[outs][1]};
-            int rc = launch_resident(s->dtype, s->L, u, v, m, s->p, s->boundary == GS_BOUNDARY_HELD, s->t,
+            Params p = s->p;
+            if (p.arith != GS_ARITH_IEEE) p.io = (i > 0 ? 1 : 0) | (i + m < n ? 2 : 0);
+            int rc = launch_resident(s->dtype, s->L, u, v, m, p, s->boundary == GS_BOUNDARY_HELD, s->t,
                                      (unsigned*)(s->d_err + 4), s->d_err, s->timeout_ns, s->stream);
             if (rc) return rc;
             s->launches += 1;

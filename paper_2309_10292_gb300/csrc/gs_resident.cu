@@ -13,6 +13,8 @@
 //   FP32  L = 32: 28.8 -> 1.8   64: 30.9 -> 2.2   96: 30.9 -> 3.9
 //         L = 128: 33.0 -> 6.4  160: 34.9 -> 10.4  200: 41.4 -> 25  256: 53.3 -> 48
 //   FP64  L = 64: 119 -> 13.4   128: 121 -> 93.7   256: 744 -> 736 (FP64 pipe)
+//   FP64 in fixed point with a remainder  L = 64: 29.5 -> 3.8   128: 29.5 -> 15.2
+//   FP64 in double-single  L = 128: 23.2, in fixed point 25.9
 // Measured and not taken: columns marched in z with register planes (fewer
 // loads, but fewer groups in flight: 64^3 2.7, 128^3 7.2 us), and x neighbours
 // from adjacent lanes (2.4 and 6.7 us: the shuffles wait for the loads).
@@ -24,7 +26,7 @@
 
 namespace gs {
 
-template <typename T>
+template <typename T, int AR>
 struct ResArgs {
     T *u0, *v0;         // the set holding the state before the first step
     T *u1, *v1;         // the other set
@@ -32,14 +34,19 @@ struct ResArgs {
     int n;              // steps
     int64_t t;          // step index of the first one
     uint64_t seed;
-    GsCoef<T> c;
+    ResCoef<T, AR> c;
+    int io;             // AR > 0: bit 0 the input holds packed values, bit 1 write packed values
     unsigned* bar;      // [arrivals, CTAs done], zero between launches
     int* err;
     uint64_t timeout_ns;
 };
 
-template <typename T, int V, bool NOISE, bool HELD, int MAXT>
-__global__ void __launch_bounds__(MAXT, 1) gs_resident_kernel(const ResArgs<T> a)
+// AR > 0 (FP64 fields, periodic): the fields are converted to packed values in
+// place before the first step, stay packed between the steps, and the last
+// step writes FP64 values (a call of several launches converts only at its
+// ends, see io).
+template <typename T, int V, bool NOISE, bool HELD, int AR, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) gs_resident_kernel(const ResArgs<T, AR> a)
 {
     const int L = a.L, tid = threadIdx.x;
     // this CTA's rows: a brick (a y range times a z range), or with ny = 0 a
@@ -60,15 +67,27 @@ __global__ void __launch_bounds__(MAXT, 1) gs_resident_kernel(const ResArgs<T> a
         r.ys = r0 - r.zs * L;
     }
     const ResWalk<V> w(r, tid);
-    for (int s = 0; s < a.n; ++s) {
-        const GsKeys k = NOISE ? gs_step_keys(a.seed, a.t + s) : GsKeys{0, 0};
-        const bool even = (s & 1) == 0;
-        res_rows<T, V, NOISE, HELD>(r, w, even ? a.u0 : a.u1, even ? a.v0 : a.v1, even ? a.u1 : a.u0,
-                                    even ? a.v1 : a.v0, a.c, k, tid);
-        if (s + 1 < a.n && res_grid_sync(a.bar, (unsigned)(s + 1) * gridDim.x, a.err, a.timeout_ns)) break;
+    unsigned met = 0;  // barriers passed
+    auto meet = [&]() { return res_grid_sync(a.bar, ++met * gridDim.x, a.err, a.timeout_ns); };
+    bool stop = false, in_range = true;
+    if constexpr (AR > 0) {
+        if (!(a.io & 1)) {
+            in_range = res_pack_rows<V, AR>(r, w, a.u0, a.v0, tid);
+            stop = meet();
+        }
     }
+    for (int s = 0; s < a.n && !stop; ++s) {
+        const GsKeys k = NOISE ? gs_step_keys(a.seed, a.t + s) : GsKeys{0, 0};
+        const bool even = (s & 1) == 0, last = s + 1 == a.n;
+        const uint32_t rng = res_rows<T, V, NOISE, HELD, AR>(r, w, even ? a.u0 : a.u1, even ? a.v0 : a.v1,
+                                                             even ? a.u1 : a.u0, even ? a.v1 : a.v0, a.c, k, tid,
+                                                             AR > 0 && last && !(a.io & 2));
+        if (AR == 3) in_range &= !fxf_range_bad(rng);
+        if (!last) stop = meet();
+    }
+    if (AR >= 2 && !in_range) gs_report(a.err, GS_DERR_RANGE);
     // the last CTA to finish zeroes both words for the next launch
-    if (a.n > 1 && tid == 0) {
+    if (met && tid == 0) {
         __threadfence();
         if (atomicAdd(&a.bar[1], 1u) == gridDim.x - 1) {
             a.bar[0] = 0;
@@ -77,13 +96,22 @@ __global__ void __launch_bounds__(MAXT, 1) gs_resident_kernel(const ResArgs<T> a
     }
 }
 
-template <typename T, int V, bool NOISE, bool HELD>
+template <typename T, int AR>
+static ResCoef<T, AR> res_coef(const Params& p)
+{
+    if constexpr (AR == 0) return gs_make_coef<T>(p.Du, p.Dv, p.F, p.k, p.dt, p.noise);
+    if constexpr (AR == 1) return gs_make_coef_ds(p.Du, p.Dv, p.F, p.k, p.dt, p.noise);
+    if constexpr (AR == 2) return gs_make_coef_fx(p.Du, p.Dv, p.F, p.k, p.dt, p.noise);
+    if constexpr (AR == 3) return gs_make_coef_fxf(p.Du, p.Dv, p.F, p.k, p.dt, p.noise);
+}
+
+template <typename T, int V, bool NOISE, bool HELD, int AR = 0>
 static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, const Params& p, int64_t t,
                              unsigned* bar, int* err, uint64_t timeout_ns, cudaStream_t s)
 {
     const int nxv = L / V;
     const long long rows_all = (long long)L * L;
-    ResArgs<T> a;
+    ResArgs<T, AR> a;
     a.u0 = (T*)u[0];
     a.v0 = (T*)v[0];
     a.u1 = (T*)u[1];
@@ -92,7 +120,7 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
     // one CTA per SM, but at least 128 groups each (fewer gain nothing)
     const int cap = (int)std::min<long long>(num_sms(), std::max<long long>(1, rows_all * nxv / 128));
     int grid, rows;
-    if (V == 4) {
+    if (V == 4 || (V == 2 && AR > 0)) {
         // bricks with the smallest largest one, then the smallest halo: the
         // neighbouring rows a CTA shares come from its L1 (256^3: 48 us
         // against 72 us with runs of rows)
@@ -112,7 +140,7 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
     } else {
         // runs of rows in memory order, equal to within one row: the FP64 pipe
         // (or the scalar loads of V = 1) bounds the step, and bricks leave SMs
-        // idle (FP64 64^3 without noise: 12.2 us against 13.3 us)
+        // idle (IEEE FP64 64^3 without noise: 12.2 us against 13.3 us)
         grid = (int)std::min<long long>(cap, rows_all);
         rows = (int)((rows_all + grid - 1) / grid);
         a.ny = a.nz = 0;
@@ -127,7 +155,8 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
     a.n = n;
     a.t = t;
     a.seed = p.seed;
-    a.c = gs_make_coef<T>(p.Du, p.Dv, p.F, p.k, p.dt, p.noise);
+    a.c = res_coef<T, AR>(p);
+    a.io = p.io;
     a.bar = bar;
     a.err = err;
     a.timeout_ns = timeout_ns;
@@ -139,19 +168,27 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
     at.id = cudaLaunchAttributeCooperative;  // co-residency for the grid barrier (none in a single step)
     at.val.cooperative = 1;
     cfg.attrs = &at;
-    cfg.numAttrs = n > 1 ? 1 : 0;
-    void (*kern)(const ResArgs<T>) = gs_resident_kernel<T, V, NOISE, HELD, 1024>;
+    cfg.numAttrs = n > 1 || (AR > 0 && !(p.io & 1)) ? 1 : 0;
+    void (*kern)(const ResArgs<T, AR>) = gs_resident_kernel<T, V, NOISE, HELD, AR, 1024>;
     if constexpr (V > 1) {
-        if (!wide) kern = gs_resident_kernel<T, V, NOISE, HELD, 512>;
+        if (!wide) kern = gs_resident_kernel<T, V, NOISE, HELD, AR, 512>;
     }
     GS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, a));
     return GS_OK;
 }
 
-// Up to 256^3 this kernel is the faster one, or (FP64) as fast as the others;
-// above, the fields leave L2 and the z-march kernel's fewer loads win (FP32
-// 320^3: 92 against 90 us; 384^3: 245 against 143 us).
-bool resident_supported(int L) { return L <= 256; }
+// Up to 256^3 this kernel is the faster one, or (IEEE FP64) as fast as the
+// others; above, the fields leave L2 and the z-march kernel's fewer loads win
+// (FP32 320^3: 92 against 86 us; 384^3: 245 against 143 us).  The other FP64
+// arithmetics unpack each value at every use here and once in the z-march
+// kernel: equal at 160^3 (fixed point with a remainder 35.5 / 35.9 us; 128^3
+// 15.2 / 21.3; 192^3 58.9 / 51.0), and odd edges, which only the plain kernel
+// takes besides, gain up to about 180 (101^3 10.5 / 15.3 us, 201^3 101 / 95).
+bool resident_supported(int L, int arith)
+{
+    if (arith == GS_ARITH_IEEE) return L <= 256;
+    return L <= (L % 2 == 0 ? 160 : 180);
+}
 
 int launch_resident(int dtype, int L, void* const u[2], void* const v[2], int n, const Params& p, bool held, int64_t t,
                     unsigned* bar, int* err, uint64_t timeout_ns, cudaStream_t s)
@@ -166,9 +203,21 @@ int launch_resident(int dtype, int L, void* const u[2], void* const v[2], int n,
         if (L % 4 == 0) GS_RES(float, 4);
         GS_RES(float, 1);
     }
+#define GS_RES_AR(AR)                                                                                                   \
+    if (p.arith == AR) {                                                                                               \
+        if (L % 2 == 0)                                                                                                \
+            return noise ? resident_launch_t<double, 2, true, false, AR>(L, u, v, n, p, t, bar, err, timeout_ns, s)    \
+                         : resident_launch_t<double, 2, false, false, AR>(L, u, v, n, p, t, bar, err, timeout_ns, s);  \
+        return noise ? resident_launch_t<double, 1, true, false, AR>(L, u, v, n, p, t, bar, err, timeout_ns, s)        \
+                     : resident_launch_t<double, 1, false, false, AR>(L, u, v, n, p, t, bar, err, timeout_ns, s);      \
+    }
+    GS_RES_AR(GS_ARITH_DS)
+    GS_RES_AR(GS_ARITH_FX)
+    GS_RES_AR(GS_ARITH_FXF)
     if (L % 2 == 0) GS_RES(double, 2);
     GS_RES(double, 1);
 #undef GS_RES
+#undef GS_RES_AR
 }
 
 }  // namespace gs

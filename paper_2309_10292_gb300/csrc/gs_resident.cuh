@@ -2,7 +2,12 @@
 // per launch (single grid: gs_resident.cu, batch: gs_batch.cu).
 #pragma once
 
+#include <type_traits>
+
 #include "gs_common.cuh"
+#include "gs_ds.cuh"
+#include "gs_fx.cuh"
+#include "gs_fxf.cuh"
 
 // V cells of one 16-byte vector, or one cell (V = 1: edges L that are no
 // multiple of the vector)
@@ -45,12 +50,80 @@ struct ResWalk {
     }
 };
 
-// One step of the cells of a run.  u, v, un, vn without __restrict__: other
-// CTAs write in one step what this one reads in the next.
-template <typename T, int V, bool NOISE, bool HELD>
-GS_D void res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const T* v, T* un, T* vn, const GsCoef<T>& c,
-                   GsKeys k, int tid)
+// Coefficients of arithmetic AR (0: IEEE, 1: double-single, 2: fixed point, 3:
+// fixed point with a float remainder).
+template <typename T, int AR>
+using ResCoef = std::conditional_t<AR == 0, GsCoef<T>,
+                                   std::conditional_t<AR == 1, GsCoefDS, std::conditional_t<AR == 2, GsCoefFX, GsCoefFXF>>>;
+
+// V cells from FP64 to AR's packed values; false: a value out of its range
+template <int V, int AR>
+GS_D bool res_pack(double* x)
 {
+    bool ok = true;
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+        bool o = false;
+        if constexpr (AR == 1) x[e] = ds_pack(ds_from_double(x[e]));
+        if constexpr (AR == 2) x[e] = fx_pack(fx_from_double(x[e], o));
+        if constexpr (AR == 3) x[e] = fxf_pack(fxf_from_double(x[e], o));
+        ok &= !o;
+    }
+    return ok;
+}
+
+template <int V, int AR>
+GS_D void res_unpack(double* x)
+{
+#pragma unroll
+    for (int e = 0; e < V; ++e) {
+        if constexpr (AR == 1) x[e] = ds_to_double(ds_unpack(x[e]));
+        if constexpr (AR == 2) x[e] = fx_to_double(fx_unpack(x[e]));
+        if constexpr (AR == 3) x[e] = fxf_to_double(fxf_unpack(x[e]));
+    }
+}
+
+// One cell whose inputs are AR's packed values (the group functions' arithmetic).
+template <bool NOISE, int AR>
+GS_D void res_cell(const ResCoef<double, AR>& c, int32_t rn, double cu, double cv, double xlu, double xru, double ymu,
+                   double ypu, double pu, double nu, double xlv, double xrv, double ymv, double ypv, double pv, double nv,
+                   double& ou, double& ov, uint32_t& rng)
+{
+    if constexpr (AR == 1) {
+        GsDS a, b;
+        const GsDS su = ds_nsum(ds_unpack(xlu), ds_unpack(xru), ds_unpack(ymu), ds_unpack(ypu), ds_unpack(pu), ds_unpack(nu));
+        const GsDS sv = ds_nsum(ds_unpack(xlv), ds_unpack(xrv), ds_unpack(ymv), ds_unpack(ypv), ds_unpack(pv), ds_unpack(nv));
+        gs_update_ds<NOISE>(c, ds_unpack(cu), ds_unpack(cv), su, sv, (float)rn, a, b);
+        ou = ds_pack(a);
+        ov = ds_pack(b);
+    } else if constexpr (AR == 2) {
+        const long long su = fx_unpack(xlu) + fx_unpack(xru) + fx_unpack(ymu) + fx_unpack(ypu) + fx_unpack(pu) + fx_unpack(nu);
+        const long long sv = fx_unpack(xlv) + fx_unpack(xrv) + fx_unpack(ymv) + fx_unpack(ypv) + fx_unpack(pv) + fx_unpack(nv);
+        long long a, b;
+        gs_update_fx<NOISE>(c, fx_unpack(cu), fx_unpack(cv), su, sv, rn, a, b);
+        ou = fx_pack(a);
+        ov = fx_pack(b);
+    } else {
+        GsFxf a, b;
+        int32_t SU, SV;
+        float SLU, SLV;
+        fxf_nsum(fxf_unpack(xlu), fxf_unpack(xru), fxf_unpack(ymu), fxf_unpack(ypu), fxf_unpack(pu), fxf_unpack(nu), SU, SLU);
+        fxf_nsum(fxf_unpack(xlv), fxf_unpack(xrv), fxf_unpack(ymv), fxf_unpack(ypv), fxf_unpack(pv), fxf_unpack(nv), SV, SLV);
+        gs_update_fxf<NOISE>(c, fxf_unpack(cu), fxf_unpack(cv), SU, SLU, SV, SLV, rn, a, b, rng);
+        ou = fxf_pack(a);
+        ov = fxf_pack(b);
+    }
+}
+
+// One step of the cells of a run.  u, v, un, vn without __restrict__: other
+// CTAs write in one step what this one reads in the next.  AR > 0 (FP64): the
+// inputs are packed values, the outputs too unless `unpack`; returns the range
+// word of AR = 3 (fxf_range_bad).
+template <typename T, int V, bool NOISE, bool HELD, int AR = 0>
+GS_D uint32_t res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const T* v, T* un, T* vn,
+                       const ResCoef<T, AR>& c, GsKeys k, int tid, bool unpack = false)
+{
+    uint32_t rng = 0;
     const int L = r.L, nxv = L / V, LL = L * L, nr = r.yhi - r.ylo, ng = r.nrow * nxv;
     const uint32_t kk2 = gs_kk2(k);
     int xv = w.xv0, y = w.y0, z = w.z0;
@@ -75,7 +148,27 @@ GS_D void res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const T* v
         res_load<T, V>(v + izm, pv);
         res_load<T, V>(v + izp, nv);
         const T xlu = u[ixl], xru = u[ixr], xlv = v[ixl], xrv = v[ixr];
-        if constexpr (V == 1) {
+        if constexpr (AR > 0) {
+            if constexpr (V == 1) {
+                res_cell<NOISE, AR>(c, NOISE ? gs_noise_num((uint32_t)i, k) : 0, cu[0], cv[0], xlu, xru, ymu[0], ypu[0],
+                                    pu[0], nu[0], xlv, xrv, ymv[0], ypv[0], pv[0], nv[0], ou[0], ov[0], rng);
+            } else {
+                const uint32_t pre = NOISE ? gs_group_pre((uint32_t)i, k) : 0u;
+                if constexpr (AR == 1)
+                    gs_update_group_ds<NOISE, GsFromPacked, true>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv,
+                                                                  xlu, xru, xlv, xrv, ou, ov);
+                else if constexpr (AR == 2)
+                    gs_update_group_fx<NOISE, true>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru, xlv,
+                                                    xrv, ou, ov);
+                else
+                    gs_update_group_fxf<NOISE, true, 0>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru,
+                                                        xlv, xrv, ou, ov, rng);
+            }
+            if (unpack) {
+                res_unpack<V, AR>(ou);
+                res_unpack<V, AR>(ov);
+            }
+        } else if constexpr (V == 1) {
             const T su = gs_nsum(xlu, xru, ymu[0], ypu[0], pu[0], nu[0]);
             const T sv = gs_nsum(xlv, xrv, ymv[0], ypv[0], pv[0], nv[0]);
             gs_update<T, NOISE>(c, cu[0], cv[0], su, sv, NOISE ? (T)gs_noise_num((uint32_t)i, k) : (T)0, ou[0],
@@ -102,6 +195,33 @@ GS_D void res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const T* v
         if (xv >= nxv) { xv -= nxv; ++y; }
         if (y >= r.yhi) { y -= nr; ++z; }
     }
+    return rng;
+}
+
+// The cells of a run from FP64 to AR's packed values in place; false: some
+// value out of its range.
+template <int V, int AR>
+GS_D bool res_pack_rows(const ResRows& r, const ResWalk<V>& w, double* u, double* v, int tid)
+{
+    const int L = r.L, nxv = L / V, nr = r.yhi - r.ylo, ng = r.nrow * nxv;
+    int xv = w.xv0, y = w.y0, z = w.z0;
+    bool ok = true;
+    for (int g = tid; g < ng; g += blockDim.x) {
+        const int i = (z * L + y) * L + xv * V;
+        double a[V], b[V];
+        res_load<double, V>(u + i, a);
+        res_load<double, V>(v + i, b);
+        ok &= res_pack<V, AR>(a);
+        ok &= res_pack<V, AR>(b);
+        res_store<double, V>(u + i, a);
+        res_store<double, V>(v + i, b);
+        xv += w.dxv;
+        y += w.dy;
+        z += w.dz;
+        if (xv >= nxv) { xv -= nxv; ++y; }
+        if (y >= r.yhi) { y -= nr; ++z; }
+    }
+    return ok;
 }
 
 // Bounded grid barrier of co-resident CTAs, all threads: the CTA's stores are

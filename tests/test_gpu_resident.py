@@ -1,6 +1,6 @@
 """GPU tests of the many-steps launch that the default plan of a small grid takes.
 
-It must equal the one-thread-per-cell kernel bit for bit, whatever the edge
+It must equal the one-thread-per-cell kernel bit for bit in every arithmetic, whatever the edge
 (vector and scalar loads, one CTA to one per SM, runs of rows and bricks that
 do not divide the grid), the boundary and the grouping of steps into calls.
 """
@@ -48,6 +48,53 @@ def test_largest_grids_equal_the_plain_kernel(L, dtype):
     ref.set_plan(gs.GS_KERNEL_NAIVE)
     sim.step(5)
     ref.step(5)
+    for a, b in zip(sim.read(), ref.read()):
+        np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("arith", [gs.GS_ARITH_DS, gs.GS_ARITH_FX, gs.GS_ARITH_FXF])
+@pytest.mark.parametrize("L,noise,dt", [(1, 0.1, 1.0), (2, 0.1, 1.0), (5, 0.1, 0.5), (12, 0.0, 1.0), (33, 0.1, 1.0),
+                                        (64, 0.1, 0.5), (101, 0.1, 1.0), (160, 0.1, 1.0)])
+def test_fp64_arithmetics_equal_the_plain_kernel(L, noise, dt, arith):
+    # packed between the steps of a call, FP64 at its ends, like the plain kernel
+    rng = np.random.default_rng(L)
+    u, v = rng.uniform(0, 1, (L, L, L)), rng.uniform(0, 0.5, (L, L, L))
+    sim, ref = (make(L, "f64", noise=noise, dt=dt, seed=11) for _ in range(2))
+    ref.set_plan(gs.GS_KERNEL_NAIVE)
+    for s in (sim, ref):
+        s.arith = arith
+        s.write(u, v)
+        for n in (1, 6, 2, 0):
+            s.step(n)
+    assert gs.gs_launch_count(ref.handle) - gs.gs_launch_count(sim.handle) == 9 - 3
+    for a, b in zip(sim.read(), ref.read()):
+        np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("arith,bad", [(gs.GS_ARITH_FX, 1500.0), (gs.GS_ARITH_FXF, 5.0)])
+def test_fp64_range_is_reported(arith, bad):
+    L = 16
+    u, v = np.ones((L, L, L)), np.zeros((L, L, L))
+    u[3, 4, 5] = bad
+    sim = make(L, "f64", noise=0.0)
+    sim.arith = arith
+    sim.write(u, v)
+    sim.step(2)
+    with pytest.raises(gs.GsError) as e:
+        sim.sync()
+    assert e.value.status == gs.GS_EINVAL
+    sim.init()
+    sim.step(2)
+    sim.sync()
+
+
+def test_fp64_call_of_several_launches_stays_packed():
+    L, n = 6, 4096 + 5
+    sim, ref = (make(L, "f64", noise=0.1, seed=3) for _ in range(2))
+    ref.set_plan(gs.GS_KERNEL_NAIVE)
+    for s in (sim, ref):
+        s.arith = gs.GS_ARITH_FXF
+        s.step(n)
     for a, b in zip(sim.read(), ref.read()):
         np.testing.assert_array_equal(a, b)
 
