@@ -383,6 +383,8 @@ int gs_step(gs_sim* s, int64_t n)
         Params p = s->p;
         if (p.arith != GS_ARITH_IEEE && s->boundary == GS_BOUNDARY_PERIODIC)
             p.io = (i > first ? 1 : 0) | (i + 1 < n ? 2 : 0);
+        const bool held = s->boundary == GS_BOUNDARY_HELD;
+        p.held = held && p.arith == GS_ARITH_IEEE && s->kernel != GS_KERNEL_NAIVE;
         int rc;
         if (s->kernel != GS_KERNEL_NAIVE) {
             if (!s->maps_ok) return fail(GS_ESTATE, "tensor maps not encoded");
@@ -394,7 +396,7 @@ int gs_step(gs_sim* s, int64_t n)
         }
         if (rc) return rc;
         s->launches += 1;
-        if (s->boundary == GS_BOUNDARY_HELD) {
+        if (held && !p.held) {
             rc = launch_hold_faces(s->dtype, s->L, s->buf[in][0], s->buf[in][1], s->buf[outs][0], s->buf[outs][1],
                                    s->stream);
             if (rc) return rc;

@@ -21,6 +21,9 @@ struct Params {
     // packed values (the steps inside one gs_step call keep the fields
     // packed; the call's first step reads FP64 and its last writes FP64)
     int io = 0;
+    // IEEE arithmetic: the z-march kernel writes the cells of the outer layer
+    // back as they were (GS_BOUNDARY_HELD)
+    bool held = false;
 };
 
 // Thread-local error message + status helper.

@@ -395,7 +395,8 @@ GS_D bool zmarch_unit_seg(unsigned* tickets, const ZArgs<T>& a, ZSeg& g)
 // point, 3: fixed point with a float remainder).  IO (AR > 0): bit 0 = the
 // input fields hold that arithmetic's packed values, bit 1 = write packed
 // values; AR = 3: bit 2 = dt is 1 (its (v^2) dt product is skipped at
-// compile time).  The other arithmetics reading FP64 values convert every
+// compile time); AR = 0: bit 3 = held outer layer (its cells are written
+// back as they were).  The other arithmetics reading FP64 values convert every
 // staged plane in place once (CONV).
 template <typename T, bool NOISE, int AR, int IO = 0>
 GS_D void zmarch_body(const ZMaps& maps, const ZArgs<T>& a)
@@ -405,6 +406,7 @@ GS_D void zmarch_body(const ZMaps& maps, const ZArgs<T>& a)
     constexpr bool CONV = AR != 0 && (IO & 1) == 0;
     constexpr bool PACK = (IO & 2) != 0;
     constexpr int FXF_DT = (IO & 4) != 0 ? 1 : 2;
+    constexpr bool HELD = AR == 0 && (IO & 8) != 0;
     constexpr int V = GsVec<T>::N;
     using VT = typename GsVec<T>::type;
     extern __shared__ __align__(128) unsigned char smem[];
@@ -589,6 +591,10 @@ GS_D void zmarch_body(const ZMaps& maps, const ZArgs<T>& a)
             const int oxl = xv > 0 ? moff - 1 : a.lay.left_off + rr * V + (V - 1);
             const int oxr = has_r ? moff + V : a.lay.right_off + rr * V;
             int64_t gidx = (int64_t)(DESC ? z0 + nz - 1 : z0) * LL + (int64_t)(y0 + row) * L + x0 + xv * V;
+            // HELD: the plane, and whether the row / the group's first / last cell lie in the outer layer
+            [[maybe_unused]] int zc = DESC ? z0 + nz - 1 : z0;
+            [[maybe_unused]] const bool face_y = y0 + row == 0 || y0 + row == L - 1;
+            [[maybe_unused]] const bool face_l = x0 + xv * V == 0, face_r = x0 + xv * V + V == L;
 
             // CONV: convert this thread's cells of stage s, and the halo entries
             // only it reads, to packed double-single pairs (DS), fixed-point
@@ -702,6 +708,15 @@ GS_D void zmarch_body(const ZMaps& maps, const ZArgs<T>& a)
                     else
                         gs_update_group<T, NOISE>(a.c, pre, kk2, cu, cv, zmu, zmv, zpu, zpv, ymu, ypu, ymv, ypv, xlu,
                                                   xru, xlv, xrv, outu, outv);
+                    if constexpr (HELD) {
+                        const bool face = face_y || zc == 0 || zc == L - 1;
+#pragma unroll
+                        for (int e = 0; e < V; ++e)
+                            if (face || (e == 0 && face_l) || (e == V - 1 && face_r)) {
+                                outu[e] = cu[e];
+                                outv[e] = cv[e];
+                            }
+                    }
                     *reinterpret_cast<VT*>(a.un + gidx) = gs_pack<T>(outu);
                     *reinterpret_cast<VT*>(a.vn + gidx) = gs_pack<T>(outv);
                 }
@@ -710,6 +725,7 @@ GS_D void zmarch_body(const ZMaps& maps, const ZArgs<T>& a)
                 scp = snp;
                 advance();
                 gidx += DESC ? -LL : LL;
+                if constexpr (HELD) zc += DESC ? -1 : 1;
                 return true;
             };
 
@@ -869,6 +885,14 @@ int launch_zmarch(int dtype, int L, const ZPlan& pl, const ZMaps& maps, void* un
                   unsigned* tickets, cudaStream_t s)
 {
     const bool noise = p.noise != 0.0;
+    if (p.held) {
+        // (AR > 0: launch_hold_faces after the step instead)
+        if (dtype == GS_F32)
+            return noise ? zmarch_launch_t<float, true, 0, 8>(L, pl, maps, un, vn, p, t, d_err, timeout_ns, stall, tickets, s)
+                         : zmarch_launch_t<float, false, 0, 8>(L, pl, maps, un, vn, p, t, d_err, timeout_ns, stall, tickets, s);
+        return noise ? zmarch_launch_t<double, true, 0, 8>(L, pl, maps, un, vn, p, t, d_err, timeout_ns, stall, tickets, s)
+                     : zmarch_launch_t<double, false, 0, 8>(L, pl, maps, un, vn, p, t, d_err, timeout_ns, stall, tickets, s);
+    }
     if (dtype == GS_F32)
         return noise ? zmarch_launch_t<float, true, 0>(L, pl, maps, un, vn, p, t, d_err, timeout_ns, stall, tickets, s)
                      : zmarch_launch_t<float, false, 0>(L, pl, maps, un, vn, p, t, d_err, timeout_ns, stall, tickets, s);
