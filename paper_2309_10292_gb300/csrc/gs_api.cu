@@ -170,26 +170,58 @@ static bool finite_params(double a, double b, double c, double d, double e, doub
            std::isfinite(e) && std::isfinite(f);
 }
 
+// The z-march tile of the default plan.  The grid is cut in x into equal tiles
+// of up to 256 cells (an uneven cut idles threads: 320 = 2 x 160 runs at 86 us a
+// step in FP32, as 3 x 128 at 103 us), in y so that a tile fills its block.
+static ZPlan default_tile(const gs_sim* s)
+{
+    const int L = s->L, V = s->dtype == GS_F32 ? 4 : 2;
+    ZPlan pl;
+    pl.depth = 1;
+    const int nx = (L + 255) / 256;
+    const int even_x = ((L + nx - 1) / nx + V - 1) / V * V;
+    if (s->dtype == GS_F32 && L > 256) {
+        // about 1600 cells: 2 CTAs of 12-13 consumer warps per SM; a 6-stage
+        // ring.  us per step, noise 0.1, 128 x 8 x 32 with 4 stages -> this
+        // rule: 300^3 91 -> 76, 320^3 104 -> 86, 448^3 245 -> 219, 512^3 336 ->
+        // 326, 700^3 866 -> 833, 1024^3 2628 -> 2574
+        pl.tx = even_x;
+        pl.ty = (1536 + even_x / 2) / even_x;
+        pl.tz = 32;
+        pl.stages = 6;
+    } else if (s->dtype == GS_F64 && s->p.arith != GS_ARITH_IEEE && s->boundary == GS_BOUNDARY_PERIODIC && L > 160) {
+        // one CTA of up to 24 consumer warps per SM (72-80 registers a thread);
+        // z-chunks as long as every SM still gets a tile.  64 x 8 x 32 with 4
+        // stages -> this rule, fixed point with a remainder: 192^3 60 -> 51,
+        // 256^3 125 -> 109, 320^3 278 -> 234, 512^3 980 -> 870; double-single
+        // 256^3 210 -> 165, fixed point 222 -> 189
+        pl.tx = even_x;
+        pl.ty = 1536 / even_x;
+        const int cols = (L + pl.tx - 1) / pl.tx * ((L + pl.ty - 1) / pl.ty);
+        pl.tz = cols * ((L + 63) / 64) >= num_sms() ? 64 : cols * ((L + 31) / 32) >= num_sms() * 9 / 10 ? 32 : 16;
+        pl.stages = s->p.arith == GS_ARITH_FXF ? 6 : 4;
+    } else {
+        pl.tx = std::min(s->dtype == GS_F32 ? 128 : 64, L);
+        pl.tx -= pl.tx % V;
+        pl.ty = std::min(8, L);
+        pl.tz = std::min(32, L);
+        pl.stages = 4;
+    }
+    return pl;
+}
+
 static int default_plan(gs_sim* s)
 {
     s->auto_plan = true;
     s->auto_named = false;
+    s->kernel = GS_KERNEL_NAIVE;
     if (zmarch_supported(s->dtype, s->L)) {
-        ZPlan pl;
-        const int V = s->dtype == GS_F32 ? 4 : 2;
-        pl.tx = std::min(s->dtype == GS_F32 ? 128 : 64, s->L);
-        pl.tx -= pl.tx % V;
-        pl.ty = std::min(8, s->L);
-        pl.tz = std::min(32, s->L);
-        pl.stages = 4;
-        pl.depth = 1;
+        const ZPlan pl = default_tile(s);
         if (zmarch_validate(s->dtype, s->L, pl) == GS_OK) {
             s->zp = pl;
             s->kernel = GS_KERNEL_ZMARCH;
-            return GS_OK;
         }
     }
-    s->kernel = GS_KERNEL_NAIVE;
     return GS_OK;
 }
 
@@ -215,6 +247,14 @@ static int encode_maps(gs_sim* s)
     }
     s->maps_ok = true;
     return GS_OK;
+}
+
+// the default plan follows the arithmetic and the boundary
+static int replan(gs_sim* s)
+{
+    if (!s->auto_plan || s->auto_named) return GS_OK;
+    const int rc = default_plan(s);
+    return rc ? rc : encode_maps(s);
 }
 
 static int check_common(int L, double Du, double Dv, double F, double k, double dt, double noise,
@@ -788,7 +828,7 @@ int gs_set_boundary(gs_sim* s, int boundary)
     if (boundary == GS_BOUNDARY_HELD && s->kernel == GS_KERNEL_TBLOCK)
         return fail(GS_EINVAL, "temporal blocking supports the periodic boundary only; choose another plan first");
     s->boundary = boundary;
-    return GS_OK;
+    return replan(s);
 }
 
 int gs_set_arith(gs_sim* s, int arith)
@@ -799,7 +839,7 @@ int gs_set_arith(gs_sim* s, int arith)
     if (arith != GS_ARITH_IEEE && s->dtype != GS_F64)
         return fail(GS_EINVAL, "double-single and fixed-point arithmetic apply to FP64 fields only");
     s->p.arith = arith;
-    return GS_OK;
+    return replan(s);
 }
 
 int gs_get_arith(gs_sim* s, int* arith)

@@ -178,14 +178,23 @@ GS_D uint32_t res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const 
             gs_update_group<T, NOISE>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru, xlv, xrv,
                                       ou, ov);
         }
-        if (HELD) {
-            const bool face = y == 0 || y == L - 1 || z == 0 || z == L - 1;
+        if constexpr (HELD) {
+            // the outer layer keeps its values
+            if (y == 0 || y == L - 1 || z == 0 || z == L - 1) {
 #pragma unroll
-            for (int e = 0; e < V; ++e)
-                if (face || (e == 0 && x == 0) || (e == V - 1 && x + V == L)) {
+                for (int e = 0; e < V; ++e) {
                     ou[e] = cu[e];
                     ov[e] = cv[e];
                 }
+            }
+            if (x == 0) {
+                ou[0] = cu[0];
+                ov[0] = cv[0];
+            }
+            if (x + V == L) {
+                ou[V - 1] = cu[V - 1];
+                ov[V - 1] = cv[V - 1];
+            }
         }
         res_store<T, V>(un + i, ou);
         res_store<T, V>(vn + i, ov);

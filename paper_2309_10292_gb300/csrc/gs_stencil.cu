@@ -788,6 +788,14 @@ __global__ void __maxnreg__(72) gs_zmarch_fx_kernel(const __grid_constant__ ZMap
     zmarch_body<double, NOISE, 2, IO>(maps, a);
 }
 
+// Double-single: 72 registers with noise anyway; without, the compiler's 80
+// would leave room for 24 warps only.
+template <bool NOISE, int IO>
+__global__ void __maxnreg__(72) gs_zmarch_ds_kernel(const __grid_constant__ ZMaps maps, const ZArgs<double> a)
+{
+    zmarch_body<double, NOISE, 1, IO>(maps, a);
+}
+
 bool zmarch_supported(int dtype, int L)
 {
     const int V = dtype == GS_F32 ? 4 : 2;
@@ -868,6 +876,8 @@ static int zmarch_launch_t(int L, const ZPlan& pl, const ZMaps& maps, void* un, 
         kern = gs_zmarch_fxf_kernel<NOISE, IO>;
     else if constexpr (AR == 2)
         kern = gs_zmarch_fx_kernel<NOISE, IO>;
+    else if constexpr (AR == 1)
+        kern = gs_zmarch_ds_kernel<NOISE, IO>;
     else
         kern = gs_zmarch_kernel<T, NOISE, AR, IO>;
     GS_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
