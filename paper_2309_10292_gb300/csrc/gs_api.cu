@@ -231,11 +231,14 @@ static constexpr int kResidentSteps = 4096;
 // one of the TMA producer)
 static bool auto_is_resident(const gs_sim* s)
 {
-    if (s->fault != 0 || !resident_supported(s->L, s->p.arith)) return false;
+    if (s->fault != 0 || !resident_supported(s->dtype, s->L, s->p.arith)) return false;
     return s->p.arith == GS_ARITH_IEEE || s->boundary == GS_BOUNDARY_PERIODIC;
 }
 
 static bool runs_resident(const gs_sim* s) { return s->auto_plan && auto_is_resident(s); }
+
+// whether the default plan means the whole-row kernel instead of the plain one
+static bool auto_is_zrow(const gs_sim* s) { return s->fault == 0 && !auto_is_resident(s) && zrow_supported(s->dtype, s->L); }
 
 static int encode_maps(gs_sim* s)
 {
@@ -424,6 +427,15 @@ int gs_step(gs_sim* s, int64_t n)
         if (p.arith != GS_ARITH_IEEE && s->boundary == GS_BOUNDARY_PERIODIC)
             p.io = (i > first ? 1 : 0) | (i + 1 < n ? 2 : 0);
         const bool held = s->boundary == GS_BOUNDARY_HELD;
+        if (s->auto_plan && auto_is_zrow(s)) {
+            const int rc = launch_zrow(s->L, s->buf[in][0], s->buf[in][1], s->buf[outs][0], s->buf[outs][1], p, held, s->t,
+                                       (unsigned*)(s->d_err + 2), s->d_err, s->timeout_ns, s->stream);
+            if (rc) return rc;
+            s->launches += 1;
+            s->cur = outs;
+            s->t += 1;
+            continue;
+        }
         p.held = held && p.arith == GS_ARITH_IEEE && s->kernel != GS_KERNEL_NAIVE;
         int rc;
         if (s->kernel != GS_KERNEL_NAIVE) {
@@ -644,7 +656,7 @@ int gs_autotune(gs_sim* s, int steps_per_trial, gs_plan* results, int max_result
     std::vector<gs_plan> cand;
     cand.push_back(gs_plan{GS_KERNEL_NAIVE, 0, 0, 0, 1, 0, 0.0});
     // the default plan where it is more than its z-march tile (also tried below)
-    if (auto_is_resident(s)) cand.push_back(gs_plan{GS_KERNEL_AUTO, 0, 0, 0, 1, 0, 0.0});
+    if (auto_is_resident(s) || auto_is_zrow(s)) cand.push_back(gs_plan{GS_KERNEL_AUTO, 0, 0, 0, 1, 0, 0.0});
     const int zt[][2] = {{128, 8}, {256, 4}, {64, 16}, {128, 4}, {64, 8}, {256, 8}, {128, 16}, {32, 16}, {128, 10},
                          {128, 12}, {256, 6}};
     for (auto& t : zt)

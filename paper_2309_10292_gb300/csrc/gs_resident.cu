@@ -12,6 +12,7 @@
 // 128 x 8 x 32 launches for FP32, 64 x 8 x 32 for FP64; below: this kernel):
 //   FP32  L = 32: 28.8 -> 1.8   64: 30.9 -> 2.2   96: 30.9 -> 3.9
 //         L = 128: 33.0 -> 6.4  160: 34.9 -> 10.4  200: 41.4 -> 25  256: 53.3 -> 48
+//         (from the plain kernel) L = 150: 28.9 -> 11.5   101: 12.4 -> 6.4
 //   FP64  L = 64: 119 -> 13.4   128: 121 -> 93.7   256: 744 -> 736 (FP64 pipe)
 //   FP64 in fixed point with a remainder  L = 64: 29.5 -> 3.8   128: 29.5 -> 15.2
 //   FP64 in double-single  L = 128: 23.2, in fixed point 25.9
@@ -139,16 +140,16 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
         grid = a.ny * a.nz;
     } else {
         // runs of rows in memory order, equal to within one row: the FP64 pipe
-        // (or the scalar loads of V = 1) bounds the step, and bricks leave SMs
+        // (or the narrow loads of V < 4) bounds the step, and bricks leave SMs
         // idle (IEEE FP64 64^3 without noise: 12.2 us against 13.3 us)
         grid = (int)std::min<long long>(cap, rows_all);
         rows = (int)((rows_all + grid - 1) / grid);
         a.ny = a.nz = 0;
     }
     // 512 threads of up to 128 registers while the fields fit L2; beyond that,
-    // and with scalar loads, latency wants the 1024 (FP32 160^3: 10.4 against
+    // and with narrow loads, latency wants the 1024 (FP32 160^3: 10.4 against
     // 11.4 us; 192^3: 25.0 against 19.8 us; 101^3: 8.2 against 6.4 us)
-    const bool wide = V == 1 || 4 * (long long)sizeof(T) * L * rows_all > kResL2Fit;
+    const bool wide = V < GsVec<T>::N || 4 * (long long)sizeof(T) * L * rows_all > kResL2Fit;
     const int maxt = wide ? 1024 : 512;
     const int ng = nxv * rows, turns = (ng + maxt - 1) / maxt;
     const int threads = ((ng + turns - 1) / turns + 31) / 32 * 32;
@@ -179,15 +180,18 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
 
 // Up to 256^3 this kernel is the faster one, or (IEEE FP64) as fast as the
 // others; above, the fields leave L2 and the z-march kernel's fewer loads win
-// (FP32 320^3: 92 against 86 us; 384^3: 245 against 143 us).  The other FP64
-// arithmetics unpack each value at every use here and once in the z-march
-// kernel: equal at 160^3 (fixed point with a remainder 35.5 / 35.9 us; 128^3
-// 15.2 / 21.3; 192^3 58.9 / 51.0), and odd edges, which only the plain kernel
-// takes besides, gain up to about 180 (101^3 10.5 / 15.3 us, 201^3 101 / 95).
-bool resident_supported(int L, int arith)
+// (FP32 320^3: 92 against 86 us; 384^3: 245 against 143 us).  FP32 edges that
+// are no multiple of 4 leave it earlier, for the whole-row kernel (even: 210^3
+// 37.5 / 49.3 us, 222^3 53.0 / 49.9; odd: 201^3 42.1 / 41.2, 215^3 56.4 / 52.5).
+// The other FP64 arithmetics unpack each value at every use here and once in
+// the z-march kernel: equal at 160^3 (fixed point with a remainder 35.5 / 35.9
+// us; 128^3 15.2 / 21.3; 192^3 58.9 / 51.0), and odd edges, which only the plain
+// kernel takes besides, gain up to about 180 (101^3 10.5 / 15.3 us, 201^3 101 / 95).
+bool resident_supported(int dtype, int L, int arith)
 {
-    if (arith == GS_ARITH_IEEE) return L <= 256;
-    return L <= (L % 2 == 0 ? 160 : 180);
+    if (arith != GS_ARITH_IEEE) return L <= (L % 2 == 0 ? 160 : 180);
+    if (dtype == GS_F32 && L % 4 != 0) return L <= (L % 2 == 0 ? 218 : 202);
+    return L <= 256;
 }
 
 int launch_resident(int dtype, int L, void* const u[2], void* const v[2], int n, const Params& p, bool held, int64_t t,
@@ -201,6 +205,7 @@ int launch_resident(int dtype, int L, void* const u[2], void* const v[2], int n,
                          : resident_launch_t<T, V, false, false>(L, u, v, n, p, t, bar, err, timeout_ns, s))
     if (dtype == GS_F32) {
         if (L % 4 == 0) GS_RES(float, 4);
+        if (L % 2 == 0) GS_RES(float, 2);
         GS_RES(float, 1);
     }
 #define GS_RES_AR(AR)                                                                                                   \

@@ -9,19 +9,27 @@
 #include "gs_fx.cuh"
 #include "gs_fxf.cuh"
 
-// V cells of one 16-byte vector, or one cell (V = 1: edges L that are no
-// multiple of the vector)
+// V cells: one 16-byte vector, or fewer for edges L that are no multiple of it
+// (FP32 pairs for even L, single cells for odd L)
 template <typename T, int V>
 GS_D void res_load(const T* p, T* r)
 {
-    if constexpr (V == 1) r[0] = *p;
-    else gs_unpack<T>(*reinterpret_cast<const typename GsVec<T>::type*>(p), r);
+    if constexpr (V == 1) {
+        r[0] = *p;
+    } else if constexpr (V < GsVec<T>::N) {
+        const float2 t = *reinterpret_cast<const float2*>(p);
+        r[0] = t.x;
+        r[1] = t.y;
+    } else {
+        gs_unpack<T>(*reinterpret_cast<const typename GsVec<T>::type*>(p), r);
+    }
 }
 
 template <typename T, int V>
 GS_D void res_store(T* p, const T* r)
 {
     if constexpr (V == 1) *p = r[0];
+    else if constexpr (V < GsVec<T>::N) *reinterpret_cast<float2*>(p) = make_float2(r[0], r[1]);
     else *reinterpret_cast<typename GsVec<T>::type*>(p) = gs_pack<T>(r);
 }
 
@@ -168,11 +176,15 @@ GS_D uint32_t res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const 
                 res_unpack<V, AR>(ou);
                 res_unpack<V, AR>(ov);
             }
-        } else if constexpr (V == 1) {
-            const T su = gs_nsum(xlu, xru, ymu[0], ypu[0], pu[0], nu[0]);
-            const T sv = gs_nsum(xlv, xrv, ymv[0], ypv[0], pv[0], nv[0]);
-            gs_update<T, NOISE>(c, cu[0], cv[0], su, sv, NOISE ? (T)gs_noise_num((uint32_t)i, k) : (T)0, ou[0],
-                                ov[0]);
+        } else if constexpr (V < GsVec<T>::N) {
+            const uint32_t pre = NOISE ? gs_group_pre((uint32_t)i, k) : 0u;
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                const T su = gs_nsum(e > 0 ? cu[0] : xlu, e + 1 < V ? cu[V - 1] : xru, ymu[e], ypu[e], pu[e], nu[e]);
+                const T sv = gs_nsum(e > 0 ? cv[0] : xlv, e + 1 < V ? cv[V - 1] : xrv, ymv[e], ypv[e], pv[e], nv[e]);
+                gs_update<T, NOISE>(c, cu[e], cv[e], su, sv, NOISE ? (T)gs_group_num(pre, (uint32_t)e, kk2) : (T)0,
+                                    ou[e], ov[e]);
+            }
         } else {
             const uint32_t pre = NOISE ? gs_group_pre((uint32_t)i, k) : 0u;
             gs_update_group<T, NOISE>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru, xlv, xrv,
