@@ -13,7 +13,7 @@
 //   FP32  L = 32: 28.8 -> 1.8   64: 30.9 -> 2.2   96: 30.9 -> 3.9
 //         L = 128: 33.0 -> 6.4  160: 34.9 -> 10.4  200: 41.4 -> 25  256: 53.3 -> 48
 //         (from the plain kernel) L = 150: 28.9 -> 11.5   101: 12.4 -> 6.4
-//   FP64  L = 64: 119 -> 13.4   128: 121 -> 93.7   256: 744 -> 736 (FP64 pipe)
+//   FP64  L = 64: 119 -> 12.9   128: 121 -> 89.7   256: 744 -> 703 (FP64 pipe)
 //   FP64 in fixed point with a remainder  L = 64: 29.5 -> 3.8   128: 29.5 -> 15.2
 //   FP64 in double-single  L = 128: 23.2, in fixed point 25.9
 // Measured and not taken: columns marched in z with register planes (fewer

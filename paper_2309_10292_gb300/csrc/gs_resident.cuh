@@ -182,7 +182,7 @@ GS_D uint32_t res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const 
             for (int e = 0; e < V; ++e) {
                 const T su = gs_nsum(e > 0 ? cu[0] : xlu, e + 1 < V ? cu[V - 1] : xru, ymu[e], ypu[e], pu[e], nu[e]);
                 const T sv = gs_nsum(e > 0 ? cv[0] : xlv, e + 1 < V ? cv[V - 1] : xrv, ymv[e], ypv[e], pv[e], nv[e]);
-                gs_update<T, NOISE>(c, cu[e], cv[e], su, sv, NOISE ? (T)gs_group_num(pre, (uint32_t)e, kk2) : (T)0,
+                gs_update<T, NOISE>(c, cu[e], cv[e], su, sv, NOISE ? gs_num_as<T>(gs_group_num(pre, (uint32_t)e, kk2)) : (T)0,
                                     ou[e], ov[e]);
             }
         } else {

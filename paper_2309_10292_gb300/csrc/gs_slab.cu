@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256) gs_slab_kernel(const T* __restrict__ u, c
         T rn = (T)0;
         if (NOISE) {
             const int zg = (zg0 + zl) % L;
-            rn = (T)gs_noise_num((uint32_t)(x + L * (y + (int64_t)L * zg)), k);
+            rn = gs_num_as<T>(gs_noise_num((uint32_t)(x + L * (y + (int64_t)L * zg)), k));
         }
         T a, b;
         gs_update<T, NOISE>(c, uc, vc, su, sv, rn, a, b);

@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(256) gs_naive_kernel(const T* __restrict__ u, 
             const T su = gs_nsum(u[ixm], u[ixp], u[iym], u[iyp], u[izm], u[izp]);
             const T sv = gs_nsum(v[ixm], v[ixp], v[iym], v[iyp], v[izm], v[izp]);
             T rn = (T)0;
-            if (NOISE) rn = (T)gs_noise_num((uint32_t)i, k);
+            if (NOISE) rn = gs_num_as<T>(gs_noise_num((uint32_t)i, k));
             T a, b;
             gs_update<T, NOISE>(c, uc, vc, su, sv, rn, a, b);
             un[i] = a;
