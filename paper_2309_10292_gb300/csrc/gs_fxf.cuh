@@ -24,6 +24,7 @@
 #pragma once
 
 #include <cmath>
+#include <cstring>
 
 #include "gs_common.cuh"
 #include "gs_ds.cuh"
@@ -91,7 +92,18 @@ struct GsCoefFXF {
     int32_t KF;    // F dt in sixteenths of a unit, rounded ...
     float rF;      // ... and the rest
     int dt_one;    // dt == 1: the product (v^2) dt is skipped
+    // for the two-cell form: {c1, c1}, {-c1, -c1}, {-c2, -c2} of the five
+    // products above (a, b, f, k, n), {rF, rF}, and the packed constants
+    // -1, 1/16, 4 2^-22, -4 2^-22 (64-bit operands from the parameter space)
+    gs_f2 p1[5], m1[5], m2[5], rF2, neg, sixteenth, vs, mvs;
 };
+
+inline gs_f2 fxf_pair_host(float x)
+{
+    uint32_t b;
+    memcpy(&b, &x, 4);
+    return (gs_f2)b << 32 | b;
+}
 
 inline void fxf_split_host(double d, float& hi, float& lo)
 {
@@ -113,6 +125,17 @@ inline GsCoefFXF gs_make_coef_fxf(double Du, double Dv, double F, double k, doub
     c.KF = (int32_t)kf;
     c.rF = (float)(fs - kf);
     c.dt_one = dt == 1.0;
+    const float h[5] = {c.a1, c.b1, c.f1, c.k1, c.n1}, l[5] = {c.a2, c.b2, c.f2, c.k2, c.n2};
+    for (int i = 0; i < 5; ++i) {
+        c.p1[i] = fxf_pair_host(h[i]);
+        c.m1[i] = fxf_pair_host(-h[i]);
+        c.m2[i] = fxf_pair_host(-l[i]);
+    }
+    c.rF2 = fxf_pair_host(c.rF);
+    c.neg = fxf_pair_host(-1.0f);
+    c.sixteenth = fxf_pair_host(0.0625f);
+    c.vs = fxf_pair_host(4.0f * kFxfInvUnit);
+    c.mvs = fxf_pair_host(-4.0f * kFxfInvUnit);
     return c;
 }
 
@@ -230,6 +253,104 @@ GS_D void gs_update_fxf(const GsCoefFXF& c, GsFxf u, GsFxf v, int32_t SU, float 
     vn = fxf_finish(v, Tv, tv, rng);
 }
 
+// gs_update_fxf<NOISE, 1> of two cells with the float operations in pairs (one
+// instruction for both cells; the kernel is bound by instruction issue).  Each
+// lane does the same roundings; where the scalar form subtracts a product's
+// high part, the error is carried negated (rounding to nearest is symmetric),
+// and a - b is fma(b, -1, a).  About 60 packed instructions for two cells
+// instead of 114 scalar ones: 256 x 6 x 64 tiles, 512^3 838 -> 813 us a step with
+// noise, 764 -> 732 without; 256^3 113.5 -> 111.0 and 104.1 -> 101.1.
+template <bool NOISE>
+GS_D void gs_update_fxf2(const GsCoefFXF& c, const GsFxf (&u)[2], const GsFxf (&v)[2], const int32_t (&SU)[2],
+                         const float (&SLU)[2], const int32_t (&SV)[2], const float (&SLV)[2], const int32_t (&rnum)[2],
+                         GsFxf (&un)[2], GsFxf (&vn)[2], uint32_t& rng)
+{
+    auto i2f = [](int32_t a, int32_t b) { return gs_pk(__int2float_rn(a), __int2float_rn(b)); };
+    // (p, -e): fxf_mul with coefficient pair i
+    auto mul = [&](int i, gs_f2 xh, gs_f2 xl, gs_f2& p, gs_f2& ne) {
+        p = gs_mul2(c.p1[i], xh);
+        ne = gs_fma2(c.m1[i], xh, p);
+        ne = gs_fma2(c.m1[i], xl, ne);
+        ne = gs_fma2(c.m2[i], xh, ne);
+    };
+    // fxf_grid of (p, -e)
+    auto grid = [&](gs_f2 p, gs_f2 ne, int32_t (&K)[2], gs_f2& r) {
+        float p0, p1;
+        gs_upk(p, p0, p1);
+        K[0] = __float2int_rn(p0);
+        K[1] = __float2int_rn(p1);
+        r = gs_fma2(ne, c.neg, gs_fma2(i2f(K[0], K[1]), c.neg, p));
+    };
+    // the neighbour sums as float pairs
+    auto sum = [&](const int32_t (&S)[2], const float (&SL)[2], gs_f2& h, gs_f2& l) {
+        const float h0 = __int2float_rn(S[0]), h1 = __int2float_rn(S[1]);
+        h = gs_pk(h0, h1);
+        l = gs_add2(gs_pk(SL[0], SL[1]), i2f(S[0] - __float2int_rn(h0), S[1] - __float2int_rn(h1)));
+    };
+    gs_f2 suh, sul, svh, svl;
+    sum(SU, SLU, suh, sul);
+    sum(SV, SLV, svh, svl);
+    const gs_f2 uh = i2f(u[0].X, u[1].X), vhu = i2f(v[0].X, v[1].X);
+    const gs_f2 ul = gs_pk(u[0].l, u[1].l), vlu = gs_pk(v[0].l, v[1].l);
+    // v^2 = w1 + w2 (w1 and -w1, -w2)
+    const gs_f2 vh = gs_mul2(vhu, c.vs), vl = gs_mul2(vlu, c.vs);
+    const gs_f2 mvh = gs_mul2(vhu, c.mvs), mvl = gs_mul2(vlu, c.mvs);
+    const gs_f2 w1 = gs_mul2(vh, vh), mw1 = gs_mul2(mvh, vh);
+    gs_f2 mw2 = gs_fma2(mvh, vh, w1);
+    mw2 = gs_fma2(gs_add2(mvh, mvh), vl, mw2);
+    mw2 = gs_fma2(mvl, vl, mw2);
+    // u v^2 = q1 - nq
+    const gs_f2 q1 = gs_mul2(w1, uh);
+    gs_f2 nq = gs_fma2(mw1, uh, q1);
+    nq = gs_fma2(mw1, ul, nq);
+    nq = gs_fma2(mw2, uh, nq);
+    nq = gs_fma2(mw2, ul, nq);
+    gs_f2 p, ne, ra, rb, rq, rf, rk;
+    int32_t Ka[2], Kb[2], Kq[2], Kf[2], Kk[2];
+    mul(0, suh, sul, p, ne);   // Du / 6 S_u dt
+    grid(p, ne, Ka, ra);
+    mul(1, svh, svl, p, ne);   // Dv / 6 S_v dt
+    grid(p, ne, Kb, rb);
+    grid(q1, nq, Kq, rq);
+    mul(2, uh, ul, p, ne);     // (Du + F) u dt
+    grid(p, ne, Kf, rf);
+    mul(3, vhu, vlu, p, ne);   // (Dv + F + k) v dt
+    grid(p, ne, Kk, rk);
+    gs_f2 tu = gs_fma2(rf, c.neg, gs_add2(gs_fma2(rq, c.neg, ra), c.rF2));
+    const gs_f2 tv = gs_fma2(rk, c.neg, gs_add2(rb, rq));
+    int32_t Tu[2], Tv[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        Tu[e] = Ka[e] - Kq[e] + c.KF - Kf[e];
+        Tv[e] = Kb[e] + Kq[e] - Kk[e];
+    }
+    if (NOISE) {
+        const gs_f2 rn = i2f(rnum[0], rnum[1]);
+        const gs_f2 pn = gs_mul2(c.p1[4], rn);
+        gs_f2 en = gs_fma2(c.m1[4], rn, pn), rr;
+        en = gs_fma2(c.m2[4], rn, en);
+        int32_t Kn[2];
+        grid(pn, en, Kn, rr);
+        Tu[0] += Kn[0];
+        Tu[1] += Kn[1];
+        tu = gs_add2(tu, rr);
+    }
+    // fxf_finish of both cells
+    auto finish = [&](const GsFxf (&x)[2], gs_f2 xl, const int32_t (&T)[2], gs_f2 t, GsFxf (&r)[2]) {
+        const int32_t T0 = (T[0] + 8) >> 4, T1 = (T[1] + 8) >> 4;
+        const gs_f2 l = gs_fma2(gs_add2(i2f(T[0] - (T0 << 4), T[1] - (T1 << 4)), t), c.sixteenth, xl);
+        float l0, l1;
+        gs_upk(l, l0, l1);
+        const int32_t K0 = __float2int_rn(l0), K1 = __float2int_rn(l1);
+        gs_upk(gs_fma2(i2f(K0, K1), c.neg, l), r[0].l, r[1].l);
+        r[0].X = x[0].X + T0 + K0;
+        r[1].X = x[1].X + T1 + K1;
+        rng |= (uint32_t)(r[0].X + (1 << 24)) | (uint32_t)(r[1].X + (1 << 24));
+    };
+    finish(u, ul, Tu, tu, un);
+    finish(v, vlu, Tv, tv, vn);
+}
+
 // A 2-cell group of cells whose inputs are packed pairs (fxf_pack); writes
 // packed pairs (PACK) or FP64 values.
 template <bool NOISE, bool PACK, int DT>
@@ -238,6 +359,28 @@ GS_D void gs_update_group_fxf(const GsCoefFXF& c, uint32_t pre, uint32_t kk2, co
                               const double* ymu, const double* ypu, const double* ymv, const double* ypv,
                               double xlu, double xru, double xlv, double xrv, double* ou, double* ov, uint32_t& rng)
 {
+    if constexpr (DT == 1) {
+        GsFxf u[2], v[2], a[2], b[2];
+        int32_t SU[2], SV[2], rn[2];
+        float SLU[2], SLV[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            u[e] = fxf_unpack(cu[e]);
+            v[e] = fxf_unpack(cv[e]);
+            fxf_nsum(fxf_unpack(e > 0 ? cu[0] : xlu), fxf_unpack(e < 1 ? cu[1] : xru), fxf_unpack(ymu[e]),
+                     fxf_unpack(ypu[e]), fxf_unpack(pu[e]), fxf_unpack(nu[e]), SU[e], SLU[e]);
+            fxf_nsum(fxf_unpack(e > 0 ? cv[0] : xlv), fxf_unpack(e < 1 ? cv[1] : xrv), fxf_unpack(ymv[e]),
+                     fxf_unpack(ypv[e]), fxf_unpack(pv[e]), fxf_unpack(nv[e]), SV[e], SLV[e]);
+            rn[e] = NOISE ? gs_group_num(pre, (uint32_t)e, kk2) : 0;
+        }
+        gs_update_fxf2<NOISE>(c, u, v, SU, SLU, SV, SLV, rn, a, b, rng);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            ou[e] = PACK ? fxf_pack(a[e]) : fxf_to_double(a[e]);
+            ov[e] = PACK ? fxf_pack(b[e]) : fxf_to_double(b[e]);
+        }
+        return;
+    }
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
         const GsFxf u = fxf_unpack(cu[e]), v = fxf_unpack(cv[e]);
