@@ -20,9 +20,9 @@
 //   gs_wgrad_kernel   weight gradient: per tap, [Cin x cells] x [cells x Cout]
 //   + packing, bias-gradient, MSE-loss, Adam and weight-layout kernels.
 //
-// A CTA stages 4 output rows (y0..y0+3) of a 128-cell x segment: 6 x 3 input
-// rows with a one-cell periodic halo, and the layer's weights, in shared
-// memory with a 16-byte XOR swizzle so every ldmatrix is conflict-free.
+// A CTA keeps the layer's weights and a ring of input planes (its rows of up to
+// 128 cells with a one-cell periodic halo) in shared memory with a 16-byte XOR
+// swizzle so every ldmatrix is conflict-free.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -44,8 +44,7 @@ constexpr int kChan[kSurrLayers + 1] = {4, 32, 32, 32, 32, 32, 2};
 constexpr int kCinP[kSurrLayers] = {16, 32, 32, 32, 32, 32};
 constexpr int kCoutP[kSurrLayers] = {32, 32, 32, 32, 32, 8};
 constexpr float kFkScale = 20.f;
-constexpr int kRows = 4;          // output rows per CTA work item
-constexpr int kConvThreads = 512; // 16 warps: 4 rows x 4 segments of 32 cells
+constexpr int kConvThreads = 512; // 16 warps of two 16-cell tiles
 
 enum { EPI_FIRST = 0, EPI_HIDDEN = 1, EPI_LAST = 2, EPI_DGRAD = 3 };
 
@@ -95,6 +94,7 @@ struct ConvArgs {
     const bf16* w;      // [27][COUTP][CINP] (n-major rows of k)
     const float* bias;  // [COUTP] or null
     int N, L;
+    int rows, slots;    // output rows of a CTA's column, ring slots
     const bf16* res;    // EPI_HIDDEN: residual h_in [..][32]
     bf16* out;          // EPI_FIRST / EPI_HIDDEN: h_out [..][32]
     uint32_t* zmask;    // forward (training): ReLU mask, bit c = (pre-activation c > 0), one word a cell (or null)
@@ -108,7 +108,20 @@ struct ConvArgs {
     bf16* gz;           // EPI_DGRAD: gz = gh * mask
 };
 
-// Work item: (n, z, y-group of 4 rows, x segment).
+// A CTA advances along z through a column of R rows by SEG cells (one z plane
+// of it an item): R rows are as many 16-cell tiles as its 16 warps take at two
+// tiles each, so that the short rows of small grids fill them too.  Input
+// planes (R + 2 rows with a one-cell halo) live in a ring of 4 slots, so a
+// plane is read once per column and the next one arrives under the MMAs; rows
+// of 128 cells leave room for 3 slots, and each plane is waited for.  The
+// items, columns after columns, are shared out in equal contiguous runs.
+//
+// Bound by the mma.sync pipe (55 % busy in the hidden layers at 64^3; 34 % when
+// each item of 4 rows loaded and waited for its 18 input rows, and a row of 32
+// or 64 cells left three quarters or half of the warps idle).  us per network
+// application, before -> now: 16 grids of 32^3 2110 -> 525, 8 of 64^3 4679 -> 1856,
+// 8 of 96^3 11570 -> 6620, one of 128^3 2822 -> 1930 (252 TFLOP/s).  The sums of
+// every output run over the taps in the same order: the results are unchanged.
 template <int CINP, int COUTP, int EPI>
 __global__ void __launch_bounds__(kConvThreads, 1) gs_conv_kernel(const ConvArgs a)
 {
@@ -119,9 +132,11 @@ __global__ void __launch_bounds__(kConvThreads, 1) gs_conv_kernel(const ConvArgs
     const int SEG = L < 128 ? L : 128;
     const int HC = SEG + 2;
     const int nseg = L / SEG;
+    const int R = a.rows, RH = R + 2, S = a.slots;
+    const int ngrp = (L + R - 1) / R;
     const long long L3 = (long long)L * L * L;
     unsigned char* wsm = smem;                                      // weights
-    unsigned char* hsm = smem + 27 * COUTP * CINP * 2;              // halo [18 rows][HC cells]
+    unsigned char* hsm = smem + 27 * COUTP * CINP * 2;              // ring of planes [RH rows][HC cells]
     const uint32_t wbase = gs_smem_addr(wsm), hbase = gs_smem_addr(hsm);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
@@ -131,135 +146,168 @@ __global__ void __launch_bounds__(kConvThreads, 1) gs_conv_kernel(const ConvArgs
         cp16(wbase + swz(r, j, NCH), a.w + (size_t)r * CINP + j * 8);
     }
 
-    const int wrow = warp >> 2;           // output row within the item
-    const int wseg = (warp & 3) * 32;     // first cell of this warp's 32
-    const bool wact = wseg < SEG;
-    const int nmt = SEG - wseg >= 32 ? 2 : 1;  // m16 tiles of this warp
+    // this warp's two 16-cell tiles of a plane: row and first cell
+    const int tpr = SEG / 16;
+    int wrow[2], wcell[2];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+        wrow[mt] = (2 * warp + mt) / tpr;
+        wcell[mt] = ((2 * warp + mt) % tpr) * 16;
+        if (wrow[mt] >= R) wrow[mt] = -1;
+    }
     const int g = lane >> 2, t = lane & 3;
 
-    const long long items = (long long)a.N * L * (L / kRows) * nseg;
-    for (long long item = blockIdx.x; item < items; item += gridDim.x) {
-        const int seg = (int)(item % nseg);
-        long long r = item / nseg;
-        const int yg = (int)(r % (L / kRows));
-        r /= (L / kRows);
-        const int z = (int)(r % L);
-        const int n = (int)(r / L);
-        const int x0 = seg * SEG, y0 = yg * kRows;
-        __syncthreads();  // previous item's reads of the halo are done
-        // halo rows: yi = 0..5 -> y0 - 1 + yi, zi = 0..2 -> z - 1 + zi
-        const int hchunks = 18 * HC * NCH;
-        for (int i = tid; i < hchunks; i += kConvThreads) {
-            const int j = i % NCH;
-            const int c = (i / NCH) % HC;
-            const int hr = i / (NCH * HC);
-            const int yy = (y0 - 1 + hr % 6 + L) % L;
-            const int zz = (z - 1 + hr / 6 + L) % L;
-            const int xx = (x0 + c - 1 + L) % L;
-            const bf16* src = a.in + ((size_t)n * L3 + ((size_t)zz * L + yy) * L + xx) * CINP + j * 8;
-            cp16(hbase + swz(hr * HC + c, j, NCH), src);
-        }
-        cp_wait_all();
-        __syncthreads();
-        if (!wact) continue;
+    const long long items = (long long)a.N * ngrp * nseg * L;
+    const long long i0 = items * blockIdx.x / gridDim.x, i1 = items * (blockIdx.x + 1) / gridDim.x;
+    const int pieces = RH * HC * NCH;
+    for (long long item = i0; item < i1;) {
+        // a column: planes z0 .. z1 - 1 of it are this CTA's
+        const long long col = item / L;
+        const int z0 = (int)(item - col * L);
+        const int z1 = (int)std::min<long long>(L, z0 + (i1 - item));
+        item += z1 - z0;
+        const int seg = (int)(col % nseg);
+        const int yg = (int)((col / nseg) % ngrp);
+        const int n = (int)(col / nseg / ngrp);
+        const int x0 = seg * SEG, y0 = yg * R;
+        const bf16* in = a.in + (size_t)n * L3 * CINP;
+        // plane z (mod L) into slot z mod S (counted from z0 - 1)
+        auto load_plane = [&](int z) {
+            const int zz = (z + L) % L, slot = (z - z0 + 1) % S;
+            const uint32_t dst = hbase + (uint32_t)(slot * RH * HC * NCH * 16);
+            const bf16* pl = in + (size_t)zz * L * L * CINP;
+            for (int i = tid; i < pieces; i += kConvThreads) {
+                const int j = i % NCH, rc = i / NCH;
+                const int row = rc / HC, c = rc - row * HC;
+                int yy = y0 - 1 + row, xx = x0 + c - 1;
+                // (rows past the grid in the last group wrap as well; they are not used)
+                yy = yy < 0 ? yy + L : yy % L;
+                xx = xx < 0 ? xx + L : (xx >= L ? xx - L : xx);
+                cp16(dst + swz(rc, j, NCH), pl + ((size_t)yy * L + xx) * CINP + j * 8);
+            }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+        };
+        __syncthreads();  // the previous column's reads of the ring are done
+        load_plane(z0 - 1);
+        load_plane(z0);
+        load_plane(z0 + 1);
+        for (int z = z0; z < z1; ++z) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();
+            // 4 slots: plane z + 2 takes the slot of plane z - 2, which every
+            // warp has left behind the barrier
+            if (S > 3 && z + 1 < z1) load_plane(z + 2);
 
-        float acc[2][NT][4];
+            float acc[2][NT][4];
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
+            for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
+                for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) acc[mt][nt][i] = 0.f;
+                    for (int i = 0; i < 4; ++i) acc[mt][nt][i] = 0.f;
 
+            if (wrow[0] >= 0) {
 #pragma unroll 1
-        for (int tap = 0; tap < 27; ++tap) {
-            const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
-            const int hr = (wrow + 1 + dy) + 6 * (1 + dz);
+                for (int dzi = 0; dzi < 3; ++dzi) {
+                    const int slot = (z - z0 + dzi) % S;
+                    const uint32_t pbase = hbase + (uint32_t)(slot * RH * HC * NCH * 16);
 #pragma unroll
-            for (int kc = 0; kc < CINP / 16; ++kc) {
-                uint32_t b[NT][2];
-                if constexpr (NT == 1) {
-                    const int m = (lane >> 3) & 1;
-                    const int co = lane & 7;
-                    ldsm_x2(wbase + swz(tap * COUTP + co, kc * 2 + m, NCH), b[0][0], b[0][1]);
-                } else {
+                    for (int t9 = 0; t9 < 9; ++t9) {
+                        const int tap = 9 * dzi + t9, dy = t9 / 3 - 1, dx = t9 % 3 - 1;
 #pragma unroll
-                    for (int np = 0; np < NT; np += 2) {
-                        const int m = lane >> 3;
-                        const int co = (np + (m >> 1)) * 8 + (lane & 7);
-                        ldsm_x4(wbase + swz(tap * COUTP + co, kc * 2 + (m & 1), NCH), b[np][0], b[np][1],
-                                b[np + 1][0], b[np + 1][1]);
+                        for (int kc = 0; kc < CINP / 16; ++kc) {
+                            uint32_t b[NT][2];
+                            if constexpr (NT == 1) {
+                                const int m = (lane >> 3) & 1;
+                                const int co = lane & 7;
+                                ldsm_x2(wbase + swz(tap * COUTP + co, kc * 2 + m, NCH), b[0][0], b[0][1]);
+                            } else {
+#pragma unroll
+                                for (int np = 0; np < NT; np += 2) {
+                                    const int m = lane >> 3;
+                                    const int co = (np + (m >> 1)) * 8 + (lane & 7);
+                                    ldsm_x4(wbase + swz(tap * COUTP + co, kc * 2 + (m & 1), NCH), b[np][0], b[np][1],
+                                            b[np + 1][0], b[np + 1][1]);
+                                }
+                            }
+#pragma unroll
+                            for (int mt = 0; mt < 2; ++mt) {
+                                const int m = lane >> 3;
+                                // (a missing second tile computes the first one's row again, unused)
+                                const int row = wrow[mt] >= 0 ? wrow[mt] : wrow[0];
+                                const int cell = wcell[mt] + (lane & 7) + (m & 1) * 8;
+                                uint32_t af[4];
+                                ldsm_x4(pbase + swz((row + 1 + dy) * HC + 1 + dx + cell, kc * 2 + (m >> 1), NCH), af[0], af[1],
+                                        af[2], af[3]);
+#pragma unroll
+                                for (int nt = 0; nt < NT; ++nt) mma_bf16(acc[mt][nt], af, b[nt][0], b[nt][1]);
+                            }
+                        }
                     }
-                }
-#pragma unroll
-                for (int mt = 0; mt < 2; ++mt) {
-                    if (mt >= nmt) break;
-                    const int m = lane >> 3;
-                    const int cell = wseg + mt * 16 + (lane & 7) + (m & 1) * 8;
-                    uint32_t af[4];
-                    ldsm_x4(hbase + swz(hr * HC + 1 + dx + cell, kc * 2 + (m >> 1), NCH), af[0], af[1], af[2], af[3]);
-#pragma unroll
-                    for (int nt = 0; nt < NT; ++nt) mma_bf16(acc[mt][nt], af, b[nt][0], b[nt][1]);
                 }
             }
-        }
 
-        // epilogue
-        const int y = y0 + wrow;
+            // epilogue
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-            if (mt >= nmt) break;
+            for (int mt = 0; mt < 2; ++mt) {
+                const int y = y0 + wrow[mt];
+                if (wrow[mt] < 0 || y >= L) continue;  // (whole warps)
 #pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int x = x0 + wseg + mt * 16 + g + hh * 8;
-                const size_t cell = (size_t)n * L3 + ((size_t)z * L + y) * L + x;
-                uint32_t bits = 0;  // this thread's channels of the cell's ReLU mask
-                uint32_t mw = 0;
-                if constexpr (EPI == EPI_DGRAD) mw = a.gz ? a.mprev[cell] : 0u;
+                for (int hh = 0; hh < 2; ++hh) {
+                    const int x = x0 + wcell[mt] + g + hh * 8;
+                    const size_t cell = (size_t)n * L3 + ((size_t)z * L + y) * L + x;
+                    uint32_t bits = 0;  // this thread's channels of the cell's ReLU mask
+                    uint32_t mw = 0;
+                    if constexpr (EPI == EPI_DGRAD) mw = a.gz ? a.mprev[cell] : 0u;
 #pragma unroll
-                for (int nt = 0; nt < NT; ++nt) {
-                    const int ch = nt * 8 + 2 * t;
-                    float v0 = acc[mt][nt][2 * hh], v1 = acc[mt][nt][2 * hh + 1];
-                    if constexpr (EPI == EPI_FIRST || EPI == EPI_HIDDEN) {
-                        v0 += a.bias[ch];
-                        v1 += a.bias[ch + 1];
-                        bits |= (v0 > 0.f ? 1u : 0u) << ch;
-                        bits |= (v1 > 0.f ? 1u : 0u) << (ch + 1);
-                        float h0 = fmaxf(v0, 0.f), h1 = fmaxf(v1, 0.f);
-                        if constexpr (EPI == EPI_HIDDEN) {
-                            const __nv_bfloat162 rr = *reinterpret_cast<const __nv_bfloat162*>(a.res + cell * 32 + ch);
-                            h0 = __bfloat162float(rr.x) + h0;
-                            h1 = __bfloat162float(rr.y) + h1;
-                        }
-                        *reinterpret_cast<__nv_bfloat162*>(a.out + cell * 32 + ch) = __floats2bfloat162_rn(h0, h1);
-                    } else if constexpr (EPI == EPI_LAST) {
-                        if (ch == 0) {
-                            a.ou[cell] = a.su[cell] + (v0 + a.bias[0]);
-                            a.ov[cell] = a.sv[cell] + (v1 + a.bias[1]);
-                        }
-                    } else {  // EPI_DGRAD
-                        __nv_bfloat162* gp = reinterpret_cast<__nv_bfloat162*>(a.gh + cell * 32 + ch);
-                        if (a.gh_acc) {
-                            const __nv_bfloat162 old = *gp;
-                            v0 = __bfloat162float(old.x) + v0;
-                            v1 = __bfloat162float(old.y) + v1;
-                        }
-                        const __nv_bfloat162 gn = __floats2bfloat162_rn(v0, v1);
-                        *gp = gn;
-                        if (a.gz) {
-                            __nv_bfloat162 m = gn;
-                            if (!((mw >> ch) & 1u)) m.x = __float2bfloat16_rn(0.f);
-                            if (!((mw >> (ch + 1)) & 1u)) m.y = __float2bfloat16_rn(0.f);
-                            *reinterpret_cast<__nv_bfloat162*>(a.gz + cell * 32 + ch) = m;
+                    for (int nt = 0; nt < NT; ++nt) {
+                        const int ch = nt * 8 + 2 * t;
+                        float v0 = acc[mt][nt][2 * hh], v1 = acc[mt][nt][2 * hh + 1];
+                        if constexpr (EPI == EPI_FIRST || EPI == EPI_HIDDEN) {
+                            v0 += a.bias[ch];
+                            v1 += a.bias[ch + 1];
+                            bits |= (v0 > 0.f ? 1u : 0u) << ch;
+                            bits |= (v1 > 0.f ? 1u : 0u) << (ch + 1);
+                            float h0 = fmaxf(v0, 0.f), h1 = fmaxf(v1, 0.f);
+                            if constexpr (EPI == EPI_HIDDEN) {
+                                const __nv_bfloat162 rr = *reinterpret_cast<const __nv_bfloat162*>(a.res + cell * 32 + ch);
+                                h0 = __bfloat162float(rr.x) + h0;
+                                h1 = __bfloat162float(rr.y) + h1;
+                            }
+                            *reinterpret_cast<__nv_bfloat162*>(a.out + cell * 32 + ch) = __floats2bfloat162_rn(h0, h1);
+                        } else if constexpr (EPI == EPI_LAST) {
+                            if (ch == 0) {
+                                a.ou[cell] = a.su[cell] + (v0 + a.bias[0]);
+                                a.ov[cell] = a.sv[cell] + (v1 + a.bias[1]);
+                            }
+                        } else {  // EPI_DGRAD
+                            __nv_bfloat162* gp = reinterpret_cast<__nv_bfloat162*>(a.gh + cell * 32 + ch);
+                            if (a.gh_acc) {
+                                const __nv_bfloat162 old = *gp;
+                                v0 = __bfloat162float(old.x) + v0;
+                                v1 = __bfloat162float(old.y) + v1;
+                            }
+                            const __nv_bfloat162 gn = __floats2bfloat162_rn(v0, v1);
+                            *gp = gn;
+                            if (a.gz) {
+                                __nv_bfloat162 m = gn;
+                                if (!((mw >> ch) & 1u)) m.x = __float2bfloat16_rn(0.f);
+                                if (!((mw >> (ch + 1)) & 1u)) m.y = __float2bfloat16_rn(0.f);
+                                *reinterpret_cast<__nv_bfloat162*>(a.gz + cell * 32 + ch) = m;
+                            }
                         }
                     }
+                    if constexpr (EPI == EPI_FIRST || EPI == EPI_HIDDEN) {
+                        // the four threads of a quad hold the cell's 32 channels
+                        bits |= __shfl_xor_sync(0xffffffffu, bits, 1);
+                        bits |= __shfl_xor_sync(0xffffffffu, bits, 2);
+                        if (a.zmask && t == 0) a.zmask[cell] = bits;
+                    }
                 }
-                if constexpr (EPI == EPI_FIRST || EPI == EPI_HIDDEN) {
-                    // the four threads of a quad hold the cell's 32 channels
-                    bits |= __shfl_xor_sync(0xffffffffu, bits, 1);
-                    bits |= __shfl_xor_sync(0xffffffffu, bits, 2);
-                    if (a.zmask && t == 0) a.zmask[cell] = bits;
-                }
+            }
+            if (S == 3 && z + 1 < z1) {
+                __syncthreads();  // every warp is done with plane z - 1
+                load_plane(z + 2);
             }
         }
     }
@@ -272,10 +320,18 @@ struct WgArgs {
     const bf16* g;   // [N][L^3][GST] (first NP channels used)
     float* dw;       // [27][cin][cout] (fp32, accumulated with atomics)
     int N, L, GST, cin, cout;
+    int rows;        // rows of a CTA's column (divides L)
 };
 
-constexpr int kWgThreads = 288;  // 9 warps x 3 taps
+constexpr int kWgThreads = 864;  // one warp per tap
 
+// Like gs_conv_kernel a CTA advances along z through a column of `rows` rows,
+// with the input planes in a ring of 4 slots and the gradient planes in a ring
+// of 2, so copies run under the MMAs; every warp contracts its tap over all
+// cells of the plane (27 warps share the SM's four schedulers more evenly than
+// 9 warps of 3 taps did).  us per training step of the whole network with it and
+// gs_conv_kernel, before -> now: 16 grids of 32^3 5330 -> 1760, 8 of 64^3 12770 ->
+// 5770, 8 of 96^3 33570 -> 19260.
 template <int CINP, int NP>
 __global__ void __launch_bounds__(kWgThreads, 1) gs_wgrad_kernel(const WgArgs a)
 {
@@ -285,73 +341,91 @@ __global__ void __launch_bounds__(kWgThreads, 1) gs_wgrad_kernel(const WgArgs a)
     const int L = a.L;
     const int SEG = L < 128 ? L : 128;
     const int HC = SEG + 2;
-    const int nseg = L / SEG;
+    const int nseg = L / SEG, R = a.rows, RH = R + 2, ngrp = L / R;
     const long long L3 = (long long)L * L * L;
-    unsigned char* hsm = smem;                      // 18 halo rows of `in`
-    unsigned char* gsm = smem + 18 * HC * CINP * 2; // 4 rows of g
-    const uint32_t hbase = gs_smem_addr(hsm), gbase = gs_smem_addr(gsm);
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t plane_bytes = (uint32_t)(RH * HC * NCH * 16), g_bytes = (uint32_t)(R * SEG * GCH * 16);
+    const uint32_t hbase = gs_smem_addr(smem), gbase = hbase + 4 * plane_bytes;  // rings of in and g planes
+    const int tid = threadIdx.x, lane = tid & 31, tap = tid >> 5;
     const int g8 = lane >> 2, t4 = lane & 3;
+    const int dzi = tap / 9, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
 
-    float acc[3][MT][NT][4];
+    float acc[MT][NT][4];
 #pragma unroll
-    for (int q = 0; q < 3; ++q)
+    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
+        for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) acc[q][mt][nt][i] = 0.f;
+            for (int i = 0; i < 4; ++i) acc[mt][nt][i] = 0.f;
 
-    const long long items = (long long)a.N * L * (L / kRows) * nseg;
-    for (long long item = blockIdx.x; item < items; item += gridDim.x) {
-        const int seg = (int)(item % nseg);
-        long long r = item / nseg;
-        const int yg = (int)(r % (L / kRows));
-        r /= (L / kRows);
-        const int z = (int)(r % L);
-        const int n = (int)(r / L);
-        const int x0 = seg * SEG, y0 = yg * kRows;
-        __syncthreads();
-        for (int i = tid; i < 18 * HC * NCH; i += kWgThreads) {
-            const int j = i % NCH;
-            const int c = (i / NCH) % HC;
-            const int hr = i / (NCH * HC);
-            const int yy = (y0 - 1 + hr % 6 + L) % L;
-            const int zz = (z - 1 + hr / 6 + L) % L;
-            const int xx = (x0 + c - 1 + L) % L;
-            cp16(hbase + swz(hr * HC + c, j, NCH), a.in + ((size_t)n * L3 + ((size_t)zz * L + yy) * L + xx) * CINP + j * 8);
-        }
-        for (int i = tid; i < kRows * SEG * GCH; i += kWgThreads) {
-            const int j = i % GCH;
-            const int c = (i / GCH) % SEG;
-            const int rr = i / (GCH * SEG);
-            cp16(gbase + swz(rr * SEG + c, j, GCH),
-                 a.g + ((size_t)n * L3 + ((size_t)z * L + (y0 + rr)) * L + x0 + c) * a.GST + j * 8);
-        }
-        cp_wait_all();
-        __syncthreads();
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const int tap = warp * 3 + q;
-            const int dz = tap / 9 - 1, dy = (tap / 3) % 3 - 1, dx = tap % 3 - 1;
+    const long long items = (long long)a.N * ngrp * nseg * L;
+    const long long i0 = items * blockIdx.x / gridDim.x, i1 = items * (blockIdx.x + 1) / gridDim.x;
+    for (long long item = i0; item < i1;) {
+        const long long col = item / L;
+        const int z0 = (int)(item - col * L);
+        const int z1 = (int)std::min<long long>(L, z0 + (i1 - item));
+        item += z1 - z0;
+        const int seg = (int)(col % nseg);
+        const int yg = (int)((col / nseg) % ngrp);
+        const int n = (int)(col / nseg / ngrp);
+        const int x0 = seg * SEG, y0 = yg * R;
+        const bf16* in = a.in + (size_t)n * L3 * CINP;
+        const bf16* gr = a.g + (size_t)n * L3 * a.GST;
+        auto load_in = [&](int z) {
+            const int zz = (z + L) % L;
+            const uint32_t dst = hbase + (uint32_t)((z - z0 + 1) & 3) * plane_bytes;
+            const bf16* pl = in + (size_t)zz * L * L * CINP;
+            for (int i = tid; i < RH * HC * NCH; i += kWgThreads) {
+                const int j = i % NCH, rc = i / NCH;
+                const int row = rc / HC, c = rc - row * HC;
+                int yy = y0 - 1 + row, xx = x0 + c - 1;
+                yy = yy < 0 ? yy + L : (yy >= L ? yy - L : yy);
+                xx = xx < 0 ? xx + L : (xx >= L ? xx - L : xx);
+                cp16(dst + swz(rc, j, NCH), pl + ((size_t)yy * L + xx) * CINP + j * 8);
+            }
+        };
+        auto load_g = [&](int z) {
+            const uint32_t dst = gbase + (uint32_t)((z - z0) & 1) * g_bytes;
+            const bf16* pl = gr + ((size_t)z * L + y0) * L * a.GST;
+            for (int i = tid; i < R * SEG * GCH; i += kWgThreads) {
+                const int j = i % GCH, rc = i / GCH;
+                const int row = rc / SEG, c = rc - row * SEG;
+                cp16(dst + swz(rc, j, GCH), pl + ((size_t)row * L + x0 + c) * a.GST + j * 8);
+            }
+        };
+        __syncthreads();  // the previous column's reads of the rings are done
+        load_in(z0 - 1);
+        load_in(z0);
+        load_in(z0 + 1);
+        load_g(z0);
+        for (int z = z0; z < z1; ++z) {
+            cp_wait_all();
+            __syncthreads();
+            // the slots of input plane z - 2 and gradient plane z - 1, which
+            // every warp has left behind the barrier
+            if (z + 1 < z1) {
+                load_in(z + 2);
+                load_g(z + 1);
+            }
+            const uint32_t pbase = hbase + (uint32_t)((z - z0 + dzi) & 3) * plane_bytes;
+            const uint32_t gb = gbase + (uint32_t)((z - z0) & 1) * g_bytes;
 #pragma unroll 1
-            for (int rr = 0; rr < kRows; ++rr) {
-                const int hr = (rr + 1 + dy) + 6 * (1 + dz);
+            for (int rr = 0; rr < R; ++rr) {
+                const int hr = (rr + 1 + dy) * HC + 1 + dx;
+#pragma unroll 2
                 for (int k0 = 0; k0 < SEG; k0 += 16) {
                     // B (cells x co) from g, transposed load
                     uint32_t b[NT][2];
                     if constexpr (NT == 1) {
                         const int m = (lane >> 3) & 1;
                         const int cell = k0 + (lane & 7) + m * 8;
-                        ldsm_x2_t(gbase + swz(rr * SEG + cell, 0, GCH), b[0][0], b[0][1]);
+                        ldsm_x2_t(gb + swz(rr * SEG + cell, 0, GCH), b[0][0], b[0][1]);
                     } else {
 #pragma unroll
                         for (int np = 0; np < NT; np += 2) {
                             const int m = lane >> 3;
                             const int cell = k0 + (lane & 7) + (m & 1) * 8;
-                            ldsm_x4_t(gbase + swz(rr * SEG + cell, np + (m >> 1), GCH), b[np][0], b[np][1],
-                                      b[np + 1][0], b[np + 1][1]);
+                            ldsm_x4_t(gb + swz(rr * SEG + cell, np + (m >> 1), GCH), b[np][0], b[np][1], b[np + 1][0],
+                                      b[np + 1][1]);
                         }
                     }
 #pragma unroll
@@ -360,10 +434,9 @@ __global__ void __launch_bounds__(kWgThreads, 1) gs_wgrad_kernel(const WgArgs a)
                         const int m = lane >> 3;
                         const int cell = k0 + (lane & 7) + (m >> 1) * 8;
                         uint32_t af[4];
-                        ldsm_x4_t(hbase + swz(hr * HC + 1 + dx + cell, mt * 2 + (m & 1), NCH), af[0], af[1], af[2],
-                                  af[3]);
+                        ldsm_x4_t(pbase + swz(hr + cell, mt * 2 + (m & 1), NCH), af[0], af[1], af[2], af[3]);
 #pragma unroll
-                        for (int nt = 0; nt < NT; ++nt) mma_bf16(acc[q][mt][nt], af, b[nt][0], b[nt][1]);
+                        for (int nt = 0; nt < NT; ++nt) mma_bf16(acc[mt][nt], af, b[nt][0], b[nt][1]);
                     }
                 }
             }
@@ -371,19 +444,15 @@ __global__ void __launch_bounds__(kWgThreads, 1) gs_wgrad_kernel(const WgArgs a)
     }
     // accumulate this CTA's partial sums
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const int tap = warp * 3 + q;
+    for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
+        for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int ci = mt * 16 + g8 + (i >= 2 ? 8 : 0);
-                    const int co = nt * 8 + 2 * t4 + (i & 1);
-                    if (ci < a.cin && co < a.cout) atomicAdd(a.dw + ((size_t)tap * a.cin + ci) * a.cout + co, acc[q][mt][nt][i]);
-                }
-    }
+            for (int i = 0; i < 4; ++i) {
+                const int ci = mt * 16 + g8 + (i >= 2 ? 8 : 0);
+                const int co = nt * 8 + 2 * t4 + (i & 1);
+                if (ci < a.cin && co < a.cout) atomicAdd(a.dw + ((size_t)tap * a.cin + ci) * a.cout + co, acc[mt][nt][i]);
+            }
 }
 
 // 32-byte global store / load (p 32-byte aligned): one whole sector per thread
@@ -2045,13 +2114,16 @@ template <int CINP, int COUTP, int EPI>
 int conv_launch(gs_surr* s, ConvArgs a)
 {
     const int SEG = a.L < 128 ? a.L : 128;
-    const size_t smem = (size_t)27 * COUTP * CINP * 2 + (size_t)18 * (SEG + 2) * CINP * 2;
+    a.rows = std::min(a.L, 2 * (kConvThreads / 32) / (SEG / 16));
+    const size_t weights = (size_t)27 * COUTP * CINP * 2, plane = (size_t)(a.rows + 2) * (SEG + 2) * CINP * 2;
+    a.slots = weights + 4 * plane <= 227 * 1024 ? 4 : 3;
+    const size_t smem = weights + a.slots * plane;
     auto k = gs_conv_kernel<CINP, COUTP, EPI>;
     GS_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     GS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kConvThreads, smem));
     if (per_sm < 1) return fail(GS_EINVAL, "convolution tile does not fit on an SM");
-    const long long items = (long long)a.N * a.L * (a.L / kRows) * (a.L / SEG);
+    const long long items = (long long)a.N * a.L * ((a.L + a.rows - 1) / a.rows) * (a.L / SEG);
     const int grid = (int)std::min<long long>(items, (long long)per_sm * num_sms());
     k<<<grid, kConvThreads, smem, s->stream>>>(a);
     GS_CUDA_TRY(cudaGetLastError());
@@ -2063,13 +2135,17 @@ template <int CINP, int NP>
 int wgrad_launch(gs_surr* s, WgArgs a)
 {
     const int SEG = a.L < 128 ? a.L : 128;
-    const size_t smem = (size_t)18 * (SEG + 2) * CINP * 2 + (size_t)kRows * SEG * NP * 2;
+    // the most rows whose rings fit (L is a multiple of 16)
+    auto bytes = [&](int r) { return (size_t)4 * (r + 2) * (SEG + 2) * CINP * 2 + (size_t)2 * r * SEG * NP * 2; };
+    a.rows = 8;
+    while (bytes(a.rows) > 227 * 1024) a.rows /= 2;
+    const size_t smem = bytes(a.rows);
     auto k = gs_wgrad_kernel<CINP, NP>;
     GS_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     GS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kWgThreads, smem));
     if (per_sm < 1) return fail(GS_EINVAL, "weight-gradient tile does not fit on an SM");
-    const long long items = (long long)a.N * a.L * (a.L / kRows) * (a.L / SEG);
+    const long long items = (long long)a.N * a.L * (a.L / a.rows) * (a.L / SEG);
     const int grid = (int)std::min<long long>(items, (long long)per_sm * num_sms());
     k<<<grid, kWgThreads, smem, s->stream>>>(a);
     GS_CUDA_TRY(cudaGetLastError());
