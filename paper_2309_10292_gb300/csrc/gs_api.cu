@@ -189,12 +189,19 @@ static ZPlan default_tile(const gs_sim* s)
         pl.ty = (1536 + even_x / 2) / even_x;
         pl.tz = 32;
         pl.stages = 6;
-    } else if (s->dtype == GS_F64 && s->p.arith != GS_ARITH_IEEE && s->boundary == GS_BOUNDARY_PERIODIC && L > 160) {
+    } else if (s->dtype == GS_F64 && s->p.arith != GS_ARITH_IEEE && s->boundary == GS_BOUNDARY_HELD && L > 80 && L <= 140) {
+        // (converting every step) too few cells for the tile below: 96^3 70 -> 27
+        // us a step, 128^3 76 -> 52 (fixed point with a remainder)
+        pl.tx = even_x;
+        pl.ty = pl.tz = 8;
+        pl.stages = 4;
+    } else if (s->dtype == GS_F64 && s->p.arith != GS_ARITH_IEEE && L > (s->boundary == GS_BOUNDARY_HELD ? 140 : 160)) {
         // one CTA of up to 24 consumer warps per SM (72-80 registers a thread);
         // z-chunks as long as every SM still gets a tile.  64 x 8 x 32 with 4
         // stages -> this rule, fixed point with a remainder: 192^3 60 -> 51,
-        // 256^3 125 -> 109, 320^3 278 -> 234, 512^3 980 -> 870; double-single
-        // 256^3 210 -> 165, fixed point 222 -> 189
+        // 256^3 125 -> 109, 320^3 278 -> 234, 512^3 980 -> 870 (held: 160^3 112 ->
+        // 81, 256^3 352 -> 263, 354^3 983 -> 755); double-single 256^3 210 -> 165,
+        // fixed point 222 -> 189
         pl.tx = even_x;
         pl.ty = 1536 / even_x;
         const int cols = (L + pl.tx - 1) / pl.tx * ((L + pl.ty - 1) / pl.ty);
@@ -231,8 +238,7 @@ static constexpr int kResidentSteps = 4096;
 // one of the TMA producer)
 static bool auto_is_resident(const gs_sim* s)
 {
-    if (s->fault != 0 || !resident_supported(s->dtype, s->L, s->p.arith)) return false;
-    return s->p.arith == GS_ARITH_IEEE || s->boundary == GS_BOUNDARY_PERIODIC;
+    return s->fault == 0 && resident_supported(s->dtype, s->L, s->p.arith, s->boundary == GS_BOUNDARY_HELD);
 }
 
 static bool runs_resident(const gs_sim* s) { return s->auto_plan && auto_is_resident(s); }

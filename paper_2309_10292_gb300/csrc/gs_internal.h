@@ -104,8 +104,8 @@ int launch_zrow(int L, const void* u, const void* v, void* un, void* vn, const P
 // Many steps of a small grid in one launch (gs_resident.cu): n steps from the
 // state in (u[0], v[0]), stepping between the two sets; the result is in set
 // n & 1.  bar: two zeroed words of device memory the launch leaves zeroed.
-// p.arith other than IEEE: periodic only; packs (u[0], v[0]) in place.
-bool resident_supported(int dtype, int L, int arith);
+// p.arith other than IEEE and periodic: packs (u[0], v[0]) in place.
+bool resident_supported(int dtype, int L, int arith, bool held);
 // footprint (both buffer sets) up to which a resident step's loads are L2 hits throughout
 constexpr long long kResL2Fit = 96ll << 20;
 int launch_resident(int dtype, int L, void* const u[2], void* const v[2], int n, const Params& p, bool held, int64_t t,

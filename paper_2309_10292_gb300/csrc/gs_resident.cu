@@ -42,10 +42,10 @@ struct ResArgs {
     uint64_t timeout_ns;
 };
 
-// AR > 0 (FP64 fields, periodic): the fields are converted to packed values in
+// AR > 0 (FP64 fields): the fields are converted to packed values in
 // place before the first step, stay packed between the steps, and the last
 // step writes FP64 values (a call of several launches converts only at its
-// ends, see io).
+// ends, see io).  With HELD they are converted at every load and store.
 template <typename T, int V, bool NOISE, bool HELD, int AR, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) gs_resident_kernel(const ResArgs<T, AR> a)
 {
@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(MAXT, 1) gs_resident_kernel(const ResArgs<T, A
     unsigned met = 0;  // barriers passed
     auto meet = [&]() { return res_grid_sync(a.bar, ++met * gridDim.x, a.err, a.timeout_ns); };
     bool stop = false, in_range = true;
-    if constexpr (AR > 0) {
+    if constexpr (AR > 0 && !HELD) {
         if (!(a.io & 1)) {
             in_range = res_pack_rows<V, AR>(r, w, a.u0, a.v0, tid);
             stop = meet();
@@ -84,6 +84,7 @@ __global__ void __launch_bounds__(MAXT, 1) gs_resident_kernel(const ResArgs<T, A
                                                              even ? a.u1 : a.u0, even ? a.v1 : a.v0, a.c, k, tid,
                                                              AR > 0 && last && !(a.io & 2));
         if (AR == 3) in_range &= !fxf_range_bad(rng);
+        if (AR == 2 && HELD) in_range &= rng == 0;
         if (!last) stop = meet();
     }
     if (AR >= 2 && !in_range) gs_report(a.err, GS_DERR_RANGE);
@@ -106,7 +107,7 @@ static ResCoef<T, AR> res_coef(const Params& p)
     if constexpr (AR == 3) return gs_make_coef_fxf(p.Du, p.Dv, p.F, p.k, p.dt, p.noise);
 }
 
-template <typename T, int V, bool NOISE, bool HELD, int AR = 0>
+template <typename T, int V, bool NOISE, bool HELD, int AR>
 static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, const Params& p, int64_t t,
                              unsigned* bar, int* err, uint64_t timeout_ns, cudaStream_t s)
 {
@@ -169,7 +170,7 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
     at.id = cudaLaunchAttributeCooperative;  // co-residency for the grid barrier (none in a single step)
     at.val.cooperative = 1;
     cfg.attrs = &at;
-    cfg.numAttrs = n > 1 || (AR > 0 && !(p.io & 1)) ? 1 : 0;
+    cfg.numAttrs = n > 1 || (AR > 0 && !HELD && !(p.io & 1)) ? 1 : 0;
     void (*kern)(const ResArgs<T, AR>) = gs_resident_kernel<T, V, NOISE, HELD, AR, 1024>;
     if constexpr (V > 1) {
         if (!wide) kern = gs_resident_kernel<T, V, NOISE, HELD, AR, 512>;
@@ -187,8 +188,12 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
 // the z-march kernel: equal at 160^3 (fixed point with a remainder 35.5 / 35.9
 // us; 128^3 15.2 / 21.3; 192^3 58.9 / 51.0), and odd edges, which only the plain
 // kernel takes besides, gain up to about 180 (101^3 10.5 / 15.3 us, 201^3 101 / 95).
-bool resident_supported(int dtype, int L, int arith)
+// With the held outer layer these convert at every use: up to 80 (64^3 12.9 us
+// against 19.0 with the best z-march tile, 96^3 33.8 / 27.2), odd edges up to
+// 120 (101^3 24.5 us, plain kernel 33.2).
+bool resident_supported(int dtype, int L, int arith, bool held)
 {
+    if (arith != GS_ARITH_IEEE && held) return L <= (L % 2 == 0 ? 80 : 120);
     if (arith != GS_ARITH_IEEE) return L <= (L % 2 == 0 ? 160 : 180);
     if (dtype == GS_F32 && L % 4 != 0) return L <= (L % 2 == 0 ? 218 : 202);
     return L <= 256;
@@ -198,29 +203,26 @@ int launch_resident(int dtype, int L, void* const u[2], void* const v[2], int n,
                     unsigned* bar, int* err, uint64_t timeout_ns, cudaStream_t s)
 {
     const bool noise = p.noise != 0.0;
-#define GS_RES(T, V)                                                                                                   \
-    return noise ? (held ? resident_launch_t<T, V, true, true>(L, u, v, n, p, t, bar, err, timeout_ns, s)              \
-                         : resident_launch_t<T, V, true, false>(L, u, v, n, p, t, bar, err, timeout_ns, s))            \
-                 : (held ? resident_launch_t<T, V, false, true>(L, u, v, n, p, t, bar, err, timeout_ns, s)             \
-                         : resident_launch_t<T, V, false, false>(L, u, v, n, p, t, bar, err, timeout_ns, s))
+#define GS_RES(T, V, AR)                                                                                               \
+    return noise ? (held ? resident_launch_t<T, V, true, true, AR>(L, u, v, n, p, t, bar, err, timeout_ns, s)          \
+                         : resident_launch_t<T, V, true, false, AR>(L, u, v, n, p, t, bar, err, timeout_ns, s))        \
+                 : (held ? resident_launch_t<T, V, false, true, AR>(L, u, v, n, p, t, bar, err, timeout_ns, s)         \
+                         : resident_launch_t<T, V, false, false, AR>(L, u, v, n, p, t, bar, err, timeout_ns, s))
     if (dtype == GS_F32) {
-        if (L % 4 == 0) GS_RES(float, 4);
-        if (L % 2 == 0) GS_RES(float, 2);
-        GS_RES(float, 1);
+        if (L % 4 == 0) GS_RES(float, 4, 0);
+        if (L % 2 == 0) GS_RES(float, 2, 0);
+        GS_RES(float, 1, 0);
     }
-#define GS_RES_AR(AR)                                                                                                   \
+#define GS_RES_AR(AR)                                                                                                  \
     if (p.arith == AR) {                                                                                               \
-        if (L % 2 == 0)                                                                                                \
-            return noise ? resident_launch_t<double, 2, true, false, AR>(L, u, v, n, p, t, bar, err, timeout_ns, s)    \
-                         : resident_launch_t<double, 2, false, false, AR>(L, u, v, n, p, t, bar, err, timeout_ns, s);  \
-        return noise ? resident_launch_t<double, 1, true, false, AR>(L, u, v, n, p, t, bar, err, timeout_ns, s)        \
-                     : resident_launch_t<double, 1, false, false, AR>(L, u, v, n, p, t, bar, err, timeout_ns, s);      \
+        if (L % 2 == 0) GS_RES(double, 2, AR);                                                                         \
+        GS_RES(double, 1, AR);                                                                                         \
     }
     GS_RES_AR(GS_ARITH_DS)
     GS_RES_AR(GS_ARITH_FX)
     GS_RES_AR(GS_ARITH_FXF)
-    if (L % 2 == 0) GS_RES(double, 2);
-    GS_RES(double, 1);
+    if (L % 2 == 0) GS_RES(double, 2, 0);
+    GS_RES(double, 1, 0);
 #undef GS_RES
 #undef GS_RES_AR
 }

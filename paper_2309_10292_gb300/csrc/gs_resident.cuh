@@ -125,8 +125,10 @@ GS_D void res_cell(const ResCoef<double, AR>& c, int32_t rn, double cu, double c
 
 // One step of the cells of a run.  u, v, un, vn without __restrict__: other
 // CTAs write in one step what this one reads in the next.  AR > 0 (FP64): the
-// inputs are packed values, the outputs too unless `unpack`; returns the range
-// word of AR = 3 (fxf_range_bad).
+// inputs are packed values, the outputs too unless `unpack`; with HELD, whose
+// outer layer has to keep its FP64 values to the bit, both are FP64 values and
+// every load is converted.  Returns the range word of AR = 3 (fxf_range_bad;
+// all ones: an input out of range).
 template <typename T, int V, bool NOISE, bool HELD, int AR = 0>
 GS_D uint32_t res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const T* v, T* un, T* vn,
                        const ResCoef<T, AR>& c, GsKeys k, int tid, bool unpack = false)
@@ -155,7 +157,19 @@ GS_D uint32_t res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const 
         res_load<T, V>(v + iyp, ypv);
         res_load<T, V>(v + izm, pv);
         res_load<T, V>(v + izp, nv);
-        const T xlu = u[ixl], xru = u[ixr], xlv = v[ixl], xrv = v[ixr];
+        T xlu = u[ixl], xru = u[ixr], xlv = v[ixl], xrv = v[ixr];
+        [[maybe_unused]] T fu[V], fv[V];  // the FP64 values behind cu, cv
+        if constexpr (AR > 0 && HELD) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                fu[e] = cu[e];
+                fv[e] = cv[e];
+            }
+            bool ok = true;
+            for (T* q : {cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv}) ok &= res_pack<V, AR>(q);
+            for (T* q : {&xlu, &xru, &xlv, &xrv}) ok &= res_pack<1, AR>(q);
+            if (!ok) rng = ~0u;
+        }
         if constexpr (AR > 0) {
             if constexpr (V == 1) {
                 res_cell<NOISE, AR>(c, NOISE ? gs_noise_num((uint32_t)i, k) : 0, cu[0], cv[0], xlu, xru, ymu[0], ypu[0],
@@ -172,9 +186,16 @@ GS_D uint32_t res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const 
                     gs_update_group_fxf<NOISE, true, 0>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru,
                                                         xlv, xrv, ou, ov, rng);
             }
-            if (unpack) {
+            if (HELD || unpack) {
                 res_unpack<V, AR>(ou);
                 res_unpack<V, AR>(ov);
+            }
+            if constexpr (HELD) {
+#pragma unroll
+                for (int e = 0; e < V; ++e) {
+                    cu[e] = fu[e];
+                    cv[e] = fv[e];
+                }
             }
         } else if constexpr (V < GsVec<T>::N) {
             const uint32_t pre = NOISE ? gs_group_pre((uint32_t)i, k) : 0u;

@@ -57,26 +57,39 @@ def test_largest_grids_equal_the_plain_kernel(L, dtype):
                                         (64, 0.1, 0.5), (101, 0.1, 1.0), (160, 0.1, 1.0)])
 def test_fp64_arithmetics_equal_the_plain_kernel(L, noise, dt, arith):
     # packed between the steps of a call, FP64 at its ends, like the plain kernel
+    _fp64_against_plain(L, noise, dt, arith, False)
+
+
+@pytest.mark.parametrize("arith", [gs.GS_ARITH_DS, gs.GS_ARITH_FX, gs.GS_ARITH_FXF])
+@pytest.mark.parametrize("L,noise,dt", [(1, 0.1, 1.0), (3, 0.1, 1.0), (12, 0.0, 0.5), (33, 0.1, 1.0), (80, 0.1, 1.0),
+                                        (119, 0.0, 1.0)])
+def test_fp64_arithmetics_with_the_outer_layer_held(L, noise, dt, arith):
+    # FP64 between the steps: the outer layer keeps its values to the bit
+    _fp64_against_plain(L, noise, dt, arith, True)
+
+
+def _fp64_against_plain(L, noise, dt, arith, held):
     rng = np.random.default_rng(L)
     u, v = rng.uniform(0, 1, (L, L, L)), rng.uniform(0, 0.5, (L, L, L))
-    sim, ref = (make(L, "f64", noise=noise, dt=dt, seed=11) for _ in range(2))
+    sim, ref = (make(L, "f64", held, noise=noise, dt=dt, seed=11) for _ in range(2))
     ref.set_plan(gs.GS_KERNEL_NAIVE)
     for s in (sim, ref):
         s.arith = arith
         s.write(u, v)
         for n in (1, 6, 2, 0):
             s.step(n)
-    assert gs.gs_launch_count(ref.handle) - gs.gs_launch_count(sim.handle) == 9 - 3
+    assert gs.gs_launch_count(ref.handle) - gs.gs_launch_count(sim.handle) == (18 if held else 9) - 3
     for a, b in zip(sim.read(), ref.read()):
         np.testing.assert_array_equal(a, b)
 
 
+@pytest.mark.parametrize("held", [False, True])
 @pytest.mark.parametrize("arith,bad", [(gs.GS_ARITH_FX, 1500.0), (gs.GS_ARITH_FXF, 5.0)])
-def test_fp64_range_is_reported(arith, bad):
+def test_fp64_range_is_reported(arith, bad, held):
     L = 16
     u, v = np.ones((L, L, L)), np.zeros((L, L, L))
     u[3, 4, 5] = bad
-    sim = make(L, "f64", noise=0.0)
+    sim = make(L, "f64", held, noise=0.0)
     sim.arith = arith
     sim.write(u, v)
     sim.step(2)

@@ -35,10 +35,33 @@ def test_default_tile_equals_the_plain_kernel(L, dtype, arith, noise):
         np.testing.assert_array_equal(a, b)
 
 
+@pytest.mark.parametrize("L,arith", [(82, 1), (128, 2), (140, 3), (142, 3), (190, 1), (258, 2)])
+def test_default_tile_with_the_outer_layer_held(L, arith):
+    need_cuda()
+    out = []
+    for plain in (False, True):
+        sim = gs.GrayScott(L, dtype="f64", **dict(PAPER, noise=0.1, seed=3))
+        sim.boundary = gs.GS_BOUNDARY_HELD
+        sim.arith = arith
+        if plain:
+            sim.set_plan(gs.GS_KERNEL_NAIVE)
+        sim.step(3)
+        out.append(sim.read())
+        sim.close()
+    for a, b in zip(*out):
+        np.testing.assert_array_equal(a, b)
+
+
 def test_every_default_tile_launches():
     need_cuda()
-    for L in list(range(162, 262, 2)) + list(range(264, 520, 16)):
+    for L in list(range(82, 262, 2)) + list(range(264, 520, 16)):
         for arith in (1, 2, 3):
+            held = gs.GrayScott(L, dtype="f64", **dict(PAPER, noise=0.1 if L % 4 else 0.0, seed=3))
+            held.boundary = gs.GS_BOUNDARY_HELD
+            held.arith = arith
+            held.step(1)
+            held.sync()
+            held.close()
             sim = gs.GrayScott(L, dtype="f64", **dict(PAPER, noise=0.1 if L % 4 else 0.0, seed=3))
             sim.arith = arith
             sim.step(1)
