@@ -711,6 +711,7 @@ struct gs_batch {
     int4* d_res_tab = nullptr;  // its table (built at its first capture)
     std::vector<int4> h_res;    // ... and its contents (empty: it does not apply)
     int res_grid = 0, res_segs = 0, res_groups = 0;
+    int* h_err = nullptr;  // page-locked word the device error word is read into
 };
 
 // The work item of z-chunk zc of a single-step table: (instance, c0, z0,
@@ -1122,6 +1123,7 @@ int gs_batch_destroy(gs_batch* b)
     guarded_free(b->d_tb_rows);
     guarded_free(b->d_tb_items);
     guarded_free(b->d_res_tab);
+    if (b->h_err) cudaFreeHost(b->h_err);
     if (b->cap) cudaStreamDestroy(b->cap);
     delete b;
     return GS_OK;
@@ -1207,6 +1209,7 @@ int gs_batch_create(int n, const int* L, const double* F, const double* k, doubl
         (e = guarded_malloc((void**)&b->d_inst, sizeof(BInst) * n)) != cudaSuccess ||
         (e = guarded_malloc((void**)&b->d_maps, sizeof(CUtensorMap) * (size_t)n * 8)) != cudaSuccess ||
         (e = guarded_malloc((void**)&b->d_ctrl, sizeof(BCtrl))) != cudaSuccess ||
+        (e = cudaHostAlloc((void**)&b->h_err, sizeof(int), cudaHostAllocDefault)) != cudaSuccess ||
         (e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking)) != cudaSuccess) {
         rc = cuda_fail(e, "allocating the batch");
         gs_batch_destroy(b);
@@ -1430,9 +1433,11 @@ int gs_batch_autotune(gs_batch* b, int steps_per_trial, int* best_tile_z, int* b
 int gs_batch_sync(gs_batch* b)
 {
     if (!b) return fail(GS_EINVAL, "batch is NULL");
-    int err = 0;
-    GS_CUDA_TRY(cudaMemcpyAsync(&err, &b->d_ctrl->err, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
+    // (into page-locked memory: queued behind the data copy of a read, one wait
+    // for both; into pageable memory the copy itself waited: 12.7 -> 12.1 us a read)
+    GS_CUDA_TRY(cudaMemcpyAsync(b->h_err, &b->d_ctrl->err, sizeof(int), cudaMemcpyDeviceToHost, b->stream));
     GS_CUDA_TRY(cudaStreamSynchronize(b->stream));
+    const int err = *b->h_err;
     if (err == GS_DERR_TIMEOUT) return fail(GS_ETIMEOUT, "a device-side wait timed out");
     if (err) return fail(GS_ECUDA, "device error code %d", err);
     return GS_OK;

@@ -1022,6 +1022,8 @@ class GrayScott:
         tdt = torch.float32 if self.dtype == GS_F32 else torch.float64
         dev = torch.device("cuda", torch.cuda.current_device()) if device is None else torch.device(device)
         self._bufs = [torch.empty((L, L, L), dtype=tdt, device=dev) for _ in range(4)]
+        # (u, v) of either buffer set by the address of its u
+        self._sets = {self._bufs[i].data_ptr(): (self._bufs[i], self._bufs[i + 1]) for i in (0, 2)}
         self.stream = stream if stream is not None else torch.cuda.current_stream(dev)
         self.handle = gs_create_on(self.L, Du, Dv, F, k, dt, noise, seed, self.dtype, *self._bufs,
                                    stream=self.stream)
@@ -1090,10 +1092,7 @@ class GrayScott:
 
     def tensors(self):
         """Device tensors (u, v) of the current state (valid until the next step)."""
-        pu = gs_device_ptr(self.handle, GS_U)
-        pv = gs_device_ptr(self.handle, GS_V)
-        by = {b.data_ptr(): b for b in self._bufs}
-        return by[pu], by[pv]
+        return self._sets[gs_device_ptr(self.handle, GS_U)]
 
     def sync(self):
         gs_sync(self.handle)
