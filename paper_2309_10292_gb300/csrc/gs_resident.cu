@@ -10,12 +10,12 @@
 //
 // us per step, default plan, noise 0.1, calls of 100 steps (before: z-march
 // 128 x 8 x 32 launches for FP32, 64 x 8 x 32 for FP64; below: this kernel):
-//   FP32  L = 32: 28.8 -> 1.8   64: 30.9 -> 2.2   96: 30.9 -> 3.9
-//         L = 128: 33.0 -> 6.4  160: 34.9 -> 10.4  200: 41.4 -> 25  256: 53.3 -> 48
+//   FP32  L = 32: 28.8 -> 1.8   64: 30.9 -> 2.2   96: 30.9 -> 3.3
+//         L = 128: 33.0 -> 5.4  160: 34.9 -> 9.9  192: 41 -> 18.5  256: 53.3 -> 48.8
 //         (from the plain kernel) L = 150: 28.9 -> 11.5   101: 12.4 -> 6.4
 //   FP64  L = 64: 119 -> 12.9   128: 121 -> 89.7   256: 744 -> 703 (FP64 pipe)
-//   FP64 in fixed point with a remainder  L = 64: 29.5 -> 3.8   128: 29.5 -> 15.2
-//   FP64 in double-single  L = 128: 23.2, in fixed point 25.9
+//   FP64 in fixed point with a remainder  L = 64: 29.5 -> 3.7   128: 29.5 -> 14.8
+//   FP64 in double-single  L = 128: 23.2, in fixed point 25.3
 // Measured and not taken: columns marched in z with register planes (fewer
 // loads, but fewer groups in flight: 64^3 2.7, 128^3 7.2 us), and x neighbours
 // from adjacent lanes (2.4 and 6.7 us: the shuffles wait for the loads).
@@ -46,7 +46,7 @@ struct ResArgs {
 // place before the first step, stay packed between the steps, and the last
 // step writes FP64 values (a call of several launches converts only at its
 // ends, see io).  With HELD they are converted at every load and store.
-template <typename T, int V, bool NOISE, bool HELD, int AR, int MAXT>
+template <typename T, int V, bool NOISE, bool HELD, int AR, bool SHELL, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) gs_resident_kernel(const ResArgs<T, AR> a)
 {
     const int L = a.L, tid = threadIdx.x;
@@ -68,6 +68,7 @@ __global__ void __launch_bounds__(MAXT, 1) gs_resident_kernel(const ResArgs<T, A
         r.ys = r0 - r.zs * L;
     }
     const ResWalk<V> w(r, tid);
+    [[maybe_unused]] const ResShell q = res_shell(r);
     unsigned met = 0;  // barriers passed
     auto meet = [&]() { return res_grid_sync(a.bar, ++met * gridDim.x, a.err, a.timeout_ns); };
     bool stop = false, in_range = true;
@@ -80,12 +81,24 @@ __global__ void __launch_bounds__(MAXT, 1) gs_resident_kernel(const ResArgs<T, A
     for (int s = 0; s < a.n && !stop; ++s) {
         const GsKeys k = NOISE ? gs_step_keys(a.seed, a.t + s) : GsKeys{0, 0};
         const bool even = (s & 1) == 0, last = s + 1 == a.n;
-        const uint32_t rng = res_rows<T, V, NOISE, HELD, AR>(r, w, even ? a.u0 : a.u1, even ? a.v0 : a.v1,
-                                                             even ? a.u1 : a.u0, even ? a.v1 : a.v0, a.c, k, tid,
-                                                             AR > 0 && last && !(a.io & 2));
+        const T *u = even ? a.u0 : a.u1, *v = even ? a.v0 : a.v1;
+        T *un = even ? a.u1 : a.u0, *vn = even ? a.v1 : a.v0;
+        const bool unpack = AR > 0 && last && !(a.io & 2);
+        uint32_t rng;
+        if constexpr (SHELL) {
+            // the rows that other CTAs read, the arrival, the rest under it: a
+            // CTA that passes the barrier reads the new state of the former
+            // only, and overwrites old values that only its own rows needed
+            int2 g = make_int2(tid / (L / V), tid % (L / V));
+            rng = res_shell_rows<T, V, NOISE, HELD, AR>(q, g, q.nb, u, v, un, vn, a.c, k, unpack);
+            if (!last) res_grid_arrive(a.bar);
+            rng |= res_shell_rows<T, V, NOISE, HELD, AR>(q, g, r.nrow, u, v, un, vn, a.c, k, unpack);
+        } else {
+            rng = res_rows<T, V, NOISE, HELD, AR>(r, w, u, v, un, vn, a.c, k, tid, unpack);
+        }
         if (AR == 3) in_range &= !fxf_range_bad(rng);
         if (AR == 2 && HELD) in_range &= rng == 0;
-        if (!last) stop = meet();
+        if (!last) stop = SHELL ? res_grid_wait(a.bar, ++met * gridDim.x, a.err, a.timeout_ns) : meet();
     }
     if (AR >= 2 && !in_range) gs_report(a.err, GS_DERR_RANGE);
     // the last CTA to finish zeroes both words for the next launch
@@ -105,6 +118,17 @@ static ResCoef<T, AR> res_coef(const Params& p)
     if constexpr (AR == 1) return gs_make_coef_ds(p.Du, p.Dv, p.F, p.k, p.dt, p.noise);
     if constexpr (AR == 2) return gs_make_coef_fx(p.Du, p.Dv, p.F, p.k, p.dt, p.noise);
     if constexpr (AR == 3) return gs_make_coef_fxf(p.Du, p.Dv, p.F, p.k, p.dt, p.noise);
+}
+
+// Whether a brick steps its inner rows under the barrier.  us per step without
+// and with: FP32 64^3 2.26 / 2.29, 80^3 3.09 / 2.45, 96^3 3.89 / 3.32, 128^3 6.44 /
+// 5.40, 192^3 20.1 / 18.5, 256^3 48.8 / 48.9 (without noise 46.1 / 47.6, held 54.3 /
+// 49.4); fixed point with a remainder 64^3 3.76 / 3.68, 128^3 15.4 / 14.75, 160^3
+// 35.6 / 36.4.
+static bool shell_pays(int dtype_bytes, int L, bool held)
+{
+    if (dtype_bytes == 8) return L >= 64 && L <= 140;
+    return L >= 72 && (held || L <= 224);
 }
 
 template <typename T, int V, bool NOISE, bool HELD, int AR>
@@ -171,9 +195,13 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
     at.val.cooperative = 1;
     cfg.attrs = &at;
     cfg.numAttrs = n > 1 || (AR > 0 && !HELD && !(p.io & 1)) ? 1 : 0;
-    void (*kern)(const ResArgs<T, AR>) = gs_resident_kernel<T, V, NOISE, HELD, AR, 1024>;
+    void (*kern)(const ResArgs<T, AR>) = gs_resident_kernel<T, V, NOISE, HELD, AR, false, 1024>;
     if constexpr (V > 1) {
-        if (!wide) kern = gs_resident_kernel<T, V, NOISE, HELD, AR, 512>;
+        if (!wide) kern = gs_resident_kernel<T, V, NOISE, HELD, AR, false, 512>;
+    }
+    if constexpr (V == GsVec<T>::N && (sizeof(T) == 4 || AR > 0)) {
+        if (a.ny && n > 1 && shell_pays(sizeof(T), L, HELD))
+            kern = wide ? gs_resident_kernel<T, V, NOISE, HELD, AR, true, 1024> : gs_resident_kernel<T, V, NOISE, HELD, AR, true, 512>;
     }
     GS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, a));
     return GS_OK;

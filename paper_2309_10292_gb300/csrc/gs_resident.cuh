@@ -123,114 +123,123 @@ GS_D void res_cell(const ResCoef<double, AR>& c, int32_t rn, double cu, double c
     }
 }
 
-// One step of the cells of a run.  u, v, un, vn without __restrict__: other
+// One step of the V cells at (x, y, z).  u, v, un, vn without __restrict__: other
 // CTAs write in one step what this one reads in the next.  AR > 0 (FP64): the
 // inputs are packed values, the outputs too unless `unpack`; with HELD, whose
 // outer layer has to keep its FP64 values to the bit, both are FP64 values and
 // every load is converted.  Returns the range word of AR = 3 (fxf_range_bad;
 // all ones: an input out of range).
+template <typename T, int V, bool NOISE, bool HELD, int AR>
+GS_D uint32_t res_group(int L, int x, int y, int z, const T* u, const T* v, T* un, T* vn, const ResCoef<T, AR>& c,
+                        GsKeys k, uint32_t kk2, bool unpack)
+{
+    uint32_t rng = 0;
+    const int LL = L * L, row = (z * L + y) * L, i = row + x;  // 32 bits: L <= 256
+    const int iym = y == 0 ? i + LL - L : i - L;
+    const int iyp = y == L - 1 ? i - (LL - L) : i + L;
+    const int izm = z == 0 ? i + (L - 1) * LL : i - LL;
+    const int izp = z == L - 1 ? i - (L - 1) * LL : i + LL;
+    const int ixl = x == 0 ? row + L - 1 : i - 1;
+    const int ixr = x + V == L ? row : i + V;
+    T cu[V], cv[V], pu[V], pv[V], nu[V], nv[V], ymu[V], ypu[V], ymv[V], ypv[V], ou[V], ov[V];
+    res_load<T, V>(u + i, cu);
+    res_load<T, V>(u + iym, ymu);
+    res_load<T, V>(u + iyp, ypu);
+    res_load<T, V>(u + izm, pu);
+    res_load<T, V>(u + izp, nu);
+    res_load<T, V>(v + i, cv);
+    res_load<T, V>(v + iym, ymv);
+    res_load<T, V>(v + iyp, ypv);
+    res_load<T, V>(v + izm, pv);
+    res_load<T, V>(v + izp, nv);
+    T xlu = u[ixl], xru = u[ixr], xlv = v[ixl], xrv = v[ixr];
+    [[maybe_unused]] T fu[V], fv[V];  // the FP64 values behind cu, cv
+    if constexpr (AR > 0 && HELD) {
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            fu[e] = cu[e];
+            fv[e] = cv[e];
+        }
+        bool ok = true;
+        for (T* q : {cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv}) ok &= res_pack<V, AR>(q);
+        for (T* q : {&xlu, &xru, &xlv, &xrv}) ok &= res_pack<1, AR>(q);
+        if (!ok) rng = ~0u;
+    }
+    if constexpr (AR > 0) {
+        if constexpr (V == 1) {
+            res_cell<NOISE, AR>(c, NOISE ? gs_noise_num((uint32_t)i, k) : 0, cu[0], cv[0], xlu, xru, ymu[0], ypu[0],
+                                pu[0], nu[0], xlv, xrv, ymv[0], ypv[0], pv[0], nv[0], ou[0], ov[0], rng);
+        } else {
+            const uint32_t pre = NOISE ? gs_group_pre((uint32_t)i, k) : 0u;
+            if constexpr (AR == 1)
+                gs_update_group_ds<NOISE, GsFromPacked, true>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv,
+                                                              xlu, xru, xlv, xrv, ou, ov);
+            else if constexpr (AR == 2)
+                gs_update_group_fx<NOISE, true>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru, xlv,
+                                                xrv, ou, ov);
+            else
+                gs_update_group_fxf<NOISE, true, 0>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru,
+                                                    xlv, xrv, ou, ov, rng);
+        }
+        if (HELD || unpack) {
+            res_unpack<V, AR>(ou);
+            res_unpack<V, AR>(ov);
+        }
+        if constexpr (HELD) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                cu[e] = fu[e];
+                cv[e] = fv[e];
+            }
+        }
+    } else if constexpr (V < GsVec<T>::N) {
+        const uint32_t pre = NOISE ? gs_group_pre((uint32_t)i, k) : 0u;
+#pragma unroll
+        for (int e = 0; e < V; ++e) {
+            const T su = gs_nsum(e > 0 ? cu[0] : xlu, e + 1 < V ? cu[V - 1] : xru, ymu[e], ypu[e], pu[e], nu[e]);
+            const T sv = gs_nsum(e > 0 ? cv[0] : xlv, e + 1 < V ? cv[V - 1] : xrv, ymv[e], ypv[e], pv[e], nv[e]);
+            gs_update<T, NOISE>(c, cu[e], cv[e], su, sv, NOISE ? gs_num_as<T>(gs_group_num(pre, (uint32_t)e, kk2)) : (T)0,
+                                ou[e], ov[e]);
+        }
+    } else {
+        const uint32_t pre = NOISE ? gs_group_pre((uint32_t)i, k) : 0u;
+        gs_update_group<T, NOISE>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru, xlv, xrv,
+                                  ou, ov);
+    }
+    if constexpr (HELD) {
+        // the outer layer keeps its values
+        if (y == 0 || y == L - 1 || z == 0 || z == L - 1) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) {
+                ou[e] = cu[e];
+                ov[e] = cv[e];
+            }
+        }
+        if (x == 0) {
+            ou[0] = cu[0];
+            ov[0] = cv[0];
+        }
+        if (x + V == L) {
+            ou[V - 1] = cu[V - 1];
+            ov[V - 1] = cv[V - 1];
+        }
+    }
+    res_store<T, V>(un + i, ou);
+    res_store<T, V>(vn + i, ov);
+    return rng;
+}
+
+// One step of all cells of a run.
 template <typename T, int V, bool NOISE, bool HELD, int AR = 0>
 GS_D uint32_t res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const T* v, T* un, T* vn,
                        const ResCoef<T, AR>& c, GsKeys k, int tid, bool unpack = false)
 {
     uint32_t rng = 0;
-    const int L = r.L, nxv = L / V, LL = L * L, nr = r.yhi - r.ylo, ng = r.nrow * nxv;
+    const int L = r.L, nxv = L / V, nr = r.yhi - r.ylo, ng = r.nrow * nxv;
     const uint32_t kk2 = gs_kk2(k);
     int xv = w.xv0, y = w.y0, z = w.z0;
     for (int g = tid; g < ng; g += blockDim.x) {
-        // 32-bit indices: L <= 256
-        const int x = xv * V, row = (z * L + y) * L, i = row + x;
-        const int iym = y == 0 ? i + LL - L : i - L;
-        const int iyp = y == L - 1 ? i - (LL - L) : i + L;
-        const int izm = z == 0 ? i + (L - 1) * LL : i - LL;
-        const int izp = z == L - 1 ? i - (L - 1) * LL : i + LL;
-        const int ixl = x == 0 ? row + L - 1 : i - 1;
-        const int ixr = x + V == L ? row : i + V;
-        T cu[V], cv[V], pu[V], pv[V], nu[V], nv[V], ymu[V], ypu[V], ymv[V], ypv[V], ou[V], ov[V];
-        res_load<T, V>(u + i, cu);
-        res_load<T, V>(u + iym, ymu);
-        res_load<T, V>(u + iyp, ypu);
-        res_load<T, V>(u + izm, pu);
-        res_load<T, V>(u + izp, nu);
-        res_load<T, V>(v + i, cv);
-        res_load<T, V>(v + iym, ymv);
-        res_load<T, V>(v + iyp, ypv);
-        res_load<T, V>(v + izm, pv);
-        res_load<T, V>(v + izp, nv);
-        T xlu = u[ixl], xru = u[ixr], xlv = v[ixl], xrv = v[ixr];
-        [[maybe_unused]] T fu[V], fv[V];  // the FP64 values behind cu, cv
-        if constexpr (AR > 0 && HELD) {
-#pragma unroll
-            for (int e = 0; e < V; ++e) {
-                fu[e] = cu[e];
-                fv[e] = cv[e];
-            }
-            bool ok = true;
-            for (T* q : {cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv}) ok &= res_pack<V, AR>(q);
-            for (T* q : {&xlu, &xru, &xlv, &xrv}) ok &= res_pack<1, AR>(q);
-            if (!ok) rng = ~0u;
-        }
-        if constexpr (AR > 0) {
-            if constexpr (V == 1) {
-                res_cell<NOISE, AR>(c, NOISE ? gs_noise_num((uint32_t)i, k) : 0, cu[0], cv[0], xlu, xru, ymu[0], ypu[0],
-                                    pu[0], nu[0], xlv, xrv, ymv[0], ypv[0], pv[0], nv[0], ou[0], ov[0], rng);
-            } else {
-                const uint32_t pre = NOISE ? gs_group_pre((uint32_t)i, k) : 0u;
-                if constexpr (AR == 1)
-                    gs_update_group_ds<NOISE, GsFromPacked, true>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv,
-                                                                  xlu, xru, xlv, xrv, ou, ov);
-                else if constexpr (AR == 2)
-                    gs_update_group_fx<NOISE, true>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru, xlv,
-                                                    xrv, ou, ov);
-                else
-                    gs_update_group_fxf<NOISE, true, 0>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru,
-                                                        xlv, xrv, ou, ov, rng);
-            }
-            if (HELD || unpack) {
-                res_unpack<V, AR>(ou);
-                res_unpack<V, AR>(ov);
-            }
-            if constexpr (HELD) {
-#pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    cu[e] = fu[e];
-                    cv[e] = fv[e];
-                }
-            }
-        } else if constexpr (V < GsVec<T>::N) {
-            const uint32_t pre = NOISE ? gs_group_pre((uint32_t)i, k) : 0u;
-#pragma unroll
-            for (int e = 0; e < V; ++e) {
-                const T su = gs_nsum(e > 0 ? cu[0] : xlu, e + 1 < V ? cu[V - 1] : xru, ymu[e], ypu[e], pu[e], nu[e]);
-                const T sv = gs_nsum(e > 0 ? cv[0] : xlv, e + 1 < V ? cv[V - 1] : xrv, ymv[e], ypv[e], pv[e], nv[e]);
-                gs_update<T, NOISE>(c, cu[e], cv[e], su, sv, NOISE ? gs_num_as<T>(gs_group_num(pre, (uint32_t)e, kk2)) : (T)0,
-                                    ou[e], ov[e]);
-            }
-        } else {
-            const uint32_t pre = NOISE ? gs_group_pre((uint32_t)i, k) : 0u;
-            gs_update_group<T, NOISE>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru, xlv, xrv,
-                                      ou, ov);
-        }
-        if constexpr (HELD) {
-            // the outer layer keeps its values
-            if (y == 0 || y == L - 1 || z == 0 || z == L - 1) {
-#pragma unroll
-                for (int e = 0; e < V; ++e) {
-                    ou[e] = cu[e];
-                    ov[e] = cv[e];
-                }
-            }
-            if (x == 0) {
-                ou[0] = cu[0];
-                ov[0] = cv[0];
-            }
-            if (x + V == L) {
-                ou[V - 1] = cu[V - 1];
-                ov[V - 1] = cv[V - 1];
-            }
-        }
-        res_store<T, V>(un + i, ou);
-        res_store<T, V>(vn + i, ov);
+        rng |= res_group<T, V, NOISE, HELD, AR>(L, xv * V, y, z, u, v, un, vn, c, k, kk2, unpack);
         xv += w.dxv;
         y += w.dy;
         z += w.dz;
@@ -266,16 +275,87 @@ GS_D bool res_pack_rows(const ResRows& r, const ResWalk<V>& w, double* u, double
     return ok;
 }
 
-// Bounded grid barrier of co-resident CTAs, all threads: the CTA's stores are
-// ordered before its arrival (bar.sync makes them thread 0's predecessors),
-// every other CTA's before thread 0's acquire, and that before this CTA's
-// next loads.  `target` = arrivals after which it opens.  True: timed out.
-GS_D bool res_grid_sync(unsigned* bar, unsigned target, int* err, uint64_t timeout_ns)
+// A brick's rows with its shell (what other CTAs read) first: rows 0 .. nb - 1
+// of h x d, then the rows whose neighbours all belong to this CTA.  The walk
+// stops between the two, so that a CTA can announce its shell and go on.
+struct ResShell {
+    int L, ylo, zs, h, d, nb;
+    uint32_t inv;  // ceil(2^32 / (h - 2)): exact division of row numbers by umulhi
+};
+
+GS_D ResShell res_shell(const ResRows& r)
 {
-    __syncthreads();
+    const int h = r.yhi - r.ylo, d = r.nrow / h;
+    const int inner = h > 2 && d > 2 ? (h - 2) * (d - 2) : 0;
+    return ResShell{r.L, r.ylo, r.zs, h, d, r.nrow - inner, 0xffffffffu / (uint32_t)max(1, h - 2) + 1u};
+}
+
+// row number -> (y, z)
+GS_D void res_shell_row(const ResShell& q, int r, int& y, int& z)
+{
+    if (r >= q.nb) {
+        const int n = r - q.nb;
+        // (h = 3: inv = 2^32 does not fit)
+        const int k = q.h == 3 ? n : (int)__umulhi((uint32_t)n, q.inv);
+        y = q.ylo + 1 + n - k * (q.h - 2);
+        z = q.zs + 1 + k;
+    } else if (r < q.h || q.d == 1) {
+        y = q.ylo + r;
+        z = q.zs;
+    } else if (r < 2 * q.h) {
+        y = q.ylo + r - q.h;
+        z = q.zs + q.d - 1;
+    } else {
+        // the planes between: their first and last row (h = 1: the one row)
+        const int m = r - 2 * q.h, two = q.h > 1 ? 1 : 0;
+        z = q.zs + 1 + (m >> two);
+        y = q.ylo + ((m & two) ? q.h - 1 : 0);
+    }
+}
+
+// One step of the walk's groups (g: the next row and group of the row) up to row re.
+template <typename T, int V, bool NOISE, bool HELD, int AR>
+GS_D uint32_t res_shell_rows(const ResShell& q, int2& g, int re, const T* u, const T* v, T* un, T* vn,
+                             const ResCoef<T, AR>& c, GsKeys k, bool unpack)
+{
+    uint32_t rng = 0;
+    const int nxv = q.L / V, dr = blockDim.x / nxv, dxv = blockDim.x - dr * nxv;
+    const uint32_t kk2 = gs_kk2(k);
+    while (g.x < re) {
+        int y, z;
+        res_shell_row(q, g.x, y, z);
+        rng |= res_group<T, V, NOISE, HELD, AR>(q.L, g.y * V, y, z, u, v, un, vn, c, k, kk2, unpack);
+        g.x += dr;
+        g.y += dxv;
+        if (g.y >= nxv) { g.y -= nxv; ++g.x; }
+    }
+    return rng;
+}
+
+// Bounded grid barrier of co-resident CTAs in two halves, all threads.
+//
+// res_grid_arrive: the CTA's stores so far are ordered before its arrival (the
+// block barrier makes them thread 0's predecessors); only warp 0 waits for the
+// others, they go on with work that no other CTA sees before the next arrival.
+GS_D void res_grid_arrive(unsigned* bar)
+{
+    __syncwarp();
+    if (threadIdx.x < 32) {
+        asm volatile("barrier.cta.sync 1, %0;" ::"r"(blockDim.x) : "memory");
+        if (threadIdx.x == 0) gs_red_add_release_gpu(bar, 1u);
+        __syncwarp();
+    } else {
+        asm volatile("barrier.cta.arrive 1, %0;" ::"r"(blockDim.x) : "memory");
+    }
+}
+
+// res_grid_wait: every other CTA's arrival before thread 0's acquire, and that
+// (and this CTA's own work) before the CTA's next loads.  `target` = arrivals
+// after which it opens.  True: timed out.
+GS_D bool res_grid_wait(unsigned* bar, unsigned target, int* err, uint64_t timeout_ns)
+{
     int bad = 0;
     if (threadIdx.x == 0) {
-        gs_red_add_release_gpu(bar, 1u);
         // the counter and the target wrap modulo 2^32; their difference is exact
         if ((int)(gs_ld_acquire_gpu(bar) - target) < 0) {
             const uint64_t t0 = gs_globaltimer();
@@ -288,4 +368,11 @@ GS_D bool res_grid_sync(unsigned* bar, unsigned target, int* err, uint64_t timeo
         }
     }
     return __syncthreads_or(bad) != 0;
+}
+
+GS_D bool res_grid_sync(unsigned* bar, unsigned target, int* err, uint64_t timeout_ns)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) gs_red_add_release_gpu(bar, 1u);
+    return res_grid_wait(bar, target, err, timeout_ns);
 }
