@@ -252,9 +252,11 @@ int gs_launch_count(gs_sim* sim, int64_t* count);
 int gs_destroy(gs_sim* sim);
 
 /* Boundary treatment (GS_BOUNDARY_PERIODIC or GS_BOUNDARY_HELD).  With the
- * held outer layer every step is the chosen stencil kernel followed by a
- * copy of the six faces of the input state over the output (interior
- * results are unaffected: they read only the input state).  Temporal
+ * held outer layer the kernels write the outer cells back as they were; the
+ * plain kernel, and the z-march kernel in the FP64 arithmetics other than IEEE,
+ * are followed by a copy of the six faces instead (interior results are the
+ * same: they read only the input state).  The default plan follows the
+ * boundary and the arithmetic.  Temporal
  * blocking supports the periodic boundary only: GS_EINVAL if the current
  * plan is GS_KERNEL_TBLOCK (and gs_set_plan refuses it while held). */
 int gs_set_boundary(gs_sim* sim, int boundary);

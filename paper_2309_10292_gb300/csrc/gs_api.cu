@@ -261,8 +261,10 @@ static int encode_maps(gs_sim* s)
 // the default plan follows the arithmetic and the boundary
 static int replan(gs_sim* s)
 {
-    if (!s->auto_plan || s->auto_named) return GS_OK;
+    if (!s->auto_plan) return GS_OK;
+    const bool named = s->auto_named;
     const int rc = default_plan(s);
+    s->auto_named = named;
     return rc ? rc : encode_maps(s);
 }
 
@@ -403,13 +405,14 @@ int gs_step(gs_sim* s, int64_t n)
             if (p.arith != GS_ARITH_IEEE) p.io = (i > 0 ? 1 : 0) | (i + m < n ? 2 : 0);
             int rc = launch_resident(s->dtype, s->L, u, v, m, p, s->boundary == GS_BOUNDARY_HELD, s->t,
                                      (unsigned*)(s->d_err + 4), s->d_err, s->timeout_ns, s->stream);
+            if (rc == kResidentTooLarge) break;  // (the first launch of the call, if any)
             if (rc) return rc;
             s->launches += 1;
             s->cur = (m & 1) ? outs : in;
             s->t += m;
             i += m;
         }
-        return GS_OK;
+        if (i == n) return GS_OK;
     }
     if (s->kernel == GS_KERNEL_TBLOCK) {
         const int D = s->tp.depth;

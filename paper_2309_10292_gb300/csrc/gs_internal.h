@@ -105,6 +105,9 @@ int launch_zrow(int L, const void* u, const void* v, void* un, void* vn, const P
 // state in (u[0], v[0]), stepping between the two sets; the result is in set
 // n & 1.  bar: two zeroed words of device memory the launch leaves zeroed.
 // p.arith other than IEEE and periodic: packs (u[0], v[0]) in place.
+// Returns kResidentTooLarge (nothing launched) where its CTAs cannot all be
+// resident; the caller takes the other kernels then.
+constexpr int kResidentTooLarge = 1;
 bool resident_supported(int dtype, int L, int arith, bool held);
 // footprint (both buffer sets) up to which a resident step's loads are L2 hits throughout
 constexpr long long kResL2Fit = 96ll << 20;

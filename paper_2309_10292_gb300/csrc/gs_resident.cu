@@ -203,7 +203,13 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
         if (a.ny && n > 1 && shell_pays(sizeof(T), L, HELD))
             kern = wide ? gs_resident_kernel<T, V, NOISE, HELD, AR, true, 1024> : gs_resident_kernel<T, V, NOISE, HELD, AR, true, 512>;
     }
-    GS_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, a));
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        // (a context that may use part of the SMs only)
+        cudaGetLastError();
+        return kResidentTooLarge;
+    }
+    GS_CUDA_TRY(e);
     return GS_OK;
 }
 

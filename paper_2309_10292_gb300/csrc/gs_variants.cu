@@ -3,10 +3,12 @@
 //
 //  * held outer layer: the paper's kernel returns early for cells on the
 //    first or last layer of any axis (ghost faces filled by MPI on the full
-//    domain).  On one grid those cells keep their values.  The stencil
-//    kernels compute every cell; after each step gs_hold_faces_kernel copies
-//    the six faces of the input state over the output, which leaves interior
-//    cells exact (they read only the input state and never wrap);
+//    domain).  On one grid those cells keep their values.  The z-march (IEEE),
+//    whole-row and resident kernels write them back themselves; after a step of
+//    the plain kernel, or of the z-march kernel in the other FP64 arithmetics,
+//    gs_hold_faces_kernel copies the six faces of the input state over the
+//    output.  Interior cells are exact either way (they read only the input
+//    state and never wrap);
 //
 //  * one field without noise ("1-variable no random"):
 //      f' = f + dt (D lap f),  lap f = (s - 6 f) / 6  (Eq. 3),
