@@ -708,8 +708,7 @@ struct gs_batch {
     int tb_items_cap = 0, tb_nitems = 0, tb_items_grid = -1, tb_pe = 0, tb_grid = 0;
     // small batches under the default plan run the L2-resident kernel
     bool auto_plan = true;
-    int4* d_res_tab = nullptr;  // its table (built at its first capture)
-    std::vector<int4> h_res;    // ... and its contents (empty: it does not apply)
+    int4* d_res_tab = nullptr;  // its table (null: it does not apply)
     int res_grid = 0, res_segs = 0, res_groups = 0;
     int* h_err = nullptr;  // page-locked word the device error word is read into
 };
@@ -777,6 +776,17 @@ static void split_last(const std::vector<int4>& base, int m, int f, bool alterna
     }
 }
 
+// A table from pageable host memory, complete on the device when this returns.
+// On the batch's own stream: a plain cudaMemcpy runs on the legacy stream and may
+// return before its last part has landed, and the launches of a non-blocking
+// stream do not wait for it.
+static int upload(gs_batch* b, void* dst, const void* src, size_t bytes)
+{
+    GS_CUDA_TRY(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, b->stream));
+    GS_CUDA_TRY(cudaStreamSynchronize(b->stream));
+    return GS_OK;
+}
+
 // upload `items` as the kernel's table (growing the device buffer if needed)
 static int upload_items(gs_batch* b, const std::vector<int4>& items)
 {
@@ -787,7 +797,7 @@ static int upload_items(gs_batch* b, const std::vector<int4>& items)
         b->d_items = d;
         b->items_cap = (int)items.size();
     }
-    GS_CUDA_TRY(cudaMemcpy(b->d_items, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice));
+    if (const int rc = upload(b, b->d_items, items.data(), sizeof(int4) * items.size())) return rc;
     b->nitems = (int)items.size();
     return GS_OK;
 }
@@ -802,7 +812,7 @@ static int upload_tb_items(gs_batch* b, const std::vector<int4>& items)
         b->d_tb_items = d;
         b->tb_items_cap = (int)items.size();
     }
-    GS_CUDA_TRY(cudaMemcpy(b->d_tb_items, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice));
+    if (const int rc = upload(b, b->d_tb_items, items.data(), sizeof(int4) * items.size())) return rc;
     b->tb_nitems = (int)items.size();
     return GS_OK;
 }
@@ -829,8 +839,8 @@ static int build_tb_tables(gs_batch* b, int D)
     }
     GS_CUDA_TRY(cudaStreamSynchronize(b->stream));  // no launch still reads the old tables
     if (!b->d_tb_rows) GS_CUDA_TRY(guarded_malloc((void**)&b->d_tb_rows, sizeof(int) * b->n));
-    GS_CUDA_TRY(cudaMemcpy(b->d_tb_rows, rows.data(), sizeof(int) * b->n, cudaMemcpyHostToDevice));
-    const int rc = upload_tb_items(b, b->tb_base_items);
+    int rc = upload(b, b->d_tb_rows, rows.data(), sizeof(int) * b->n);
+    if (!rc) rc = upload_tb_items(b, b->tb_base_items);
     if (rc) return rc;
     b->tb_pe = btb_plane_elems(b->L, D);
     b->tb_items_grid = -1;
@@ -984,10 +994,12 @@ static int capture_graph(gs_batch* b, cudaGraphExec_t* exec, Launches launches)
     return fail(GS_ECUDA, "capturing the batched persistent launch failed");
 }
 
-// The resident kernel's table: equal shares of the groups of all instances,
-// cut at rows.  False if some CTA would hold more segments than fit.
-static bool plan_res_table(gs_batch* b)
+// The resident kernel's table, where the arena is small enough for it: equal
+// shares of the groups of all instances, cut at rows.  None (d_res_tab stays
+// null) if some CTA would hold more segments than fit.
+static int plan_res_table(gs_batch* b)
 {
+    if ((long long)b->arena_bytes > batch_res_bytes(b->dtype)) return GS_OK;
     const int V = b->dtype == GS_F32 ? 4 : 2;
     long long total = 0;
     for (int L : b->L) total += (long long)L * L * (L / V);
@@ -1004,7 +1016,7 @@ static bool plan_res_table(gs_batch* b)
             long long end = cta + 1 < grid ? (limit(cta) - pos + nxv - 1) / nxv : rows;
             end = std::min<long long>(rows, std::max<long long>(end, r + 1));
             if (head[cta].y == 0) head[cta].x = grid + (int)segs.size();
-            if (++head[cta].y > kResSegs) return false;
+            if (++head[cta].y > kResSegs) return GS_OK;
             segs.push_back(make_int4(i, r, (int)end - r, 0));
             r = (int)end;
         }
@@ -1014,15 +1026,15 @@ static bool plan_res_table(gs_batch* b)
     b->res_segs = (int)segs.size();
     b->res_groups = (int)((total + grid - 1) / grid);
     head.insert(head.end(), segs.begin(), segs.end());
-    b->h_res = std::move(head);
-    return true;
+    GS_CUDA_TRY(guarded_malloc((void**)&b->d_res_tab, sizeof(int4) * head.size()));
+    return upload(b, b->d_res_tab, head.data(), sizeof(int4) * head.size());
 }
 
 // Whether the default plan means the L2-resident kernel (the injected faults
 // are those of the other kernels).
 static bool auto_is_resident(const gs_batch* b)
 {
-    return b->fault == 0 && !b->h_res.empty() && (long long)b->arena_bytes <= batch_res_bytes(b->dtype);
+    return b->fault == 0 && b->d_res_tab;
 }
 
 static bool runs_resident(const gs_batch* b) { return b->auto_plan && b->depth == 1 && auto_is_resident(b); }
@@ -1030,11 +1042,6 @@ static bool runs_resident(const gs_batch* b) { return b->auto_plan && b->depth =
 template <typename T, bool NOISE>
 static int res_capture(gs_batch* b, int64_t n, cudaGraphExec_t* exec)
 {
-    if (!b->d_res_tab) {
-        const size_t bytes = sizeof(int4) * b->h_res.size();
-        GS_CUDA_TRY(guarded_malloc((void**)&b->d_res_tab, bytes));
-        GS_CUDA_TRY(cudaMemcpy(b->d_res_tab, b->h_res.data(), bytes, cudaMemcpyHostToDevice));
-    }
     const GsCoef<T> c = gs_make_coef<T>(b->Du, b->Dv, 0.0, 0.0, b->dt, b->noise);
     const BResArgs<T> a{(T*)b->arena, b->d_inst, b->d_res_tab, b->d_ctrl, n, c.Du6, c.Dv6, c.dt, c.noise24, b->timeout_ns};
     const bool wide = (long long)b->arena_bytes > kResL2Fit;  // as for a single grid
@@ -1243,14 +1250,12 @@ int gs_batch_create(int n, const int* L, const double* F, const double* k, doubl
                                (char*)b->arena + (size_t)I.off[s][1] * esz, &b->zmaps[s][i]);
     }
     if (rc == GS_OK) {
-        if ((e = cudaMemcpy(b->d_inst, b->h_inst.data(), sizeof(BInst) * n, cudaMemcpyHostToDevice)) != cudaSuccess ||
-            (e = cudaMemcpy(b->d_maps, maps.data(), sizeof(CUtensorMap) * maps.size(), cudaMemcpyHostToDevice)) !=
-                cudaSuccess ||
-            (e = cudaMemset(b->d_ctrl, 0, sizeof(BCtrl))) != cudaSuccess)
-            rc = cuda_fail(e, "uploading the batch tables");
+        if ((e = cudaMemset(b->d_ctrl, 0, sizeof(BCtrl))) != cudaSuccess) rc = cuda_fail(e, "clearing the control block");
     }
-    plan_res_table(b);
+    if (rc == GS_OK) rc = upload(b, b->d_inst, b->h_inst.data(), sizeof(BInst) * n);
+    if (rc == GS_OK) rc = upload(b, b->d_maps, maps.data(), sizeof(CUtensorMap) * maps.size());
     if (rc == GS_OK) rc = upload_items(b, b->base_items);
+    if (rc == GS_OK) rc = plan_res_table(b);
     if (rc == GS_OK) rc = gs_batch_init(b);
     if (rc != GS_OK) {
         gs_batch_destroy(b);
@@ -1524,7 +1529,7 @@ int gs_batch_set_plan(gs_batch* b, int tile_z, int stages)
         if (rc) return rc;
     }
     b->items_grid = -1;
-    GS_CUDA_TRY(cudaMemcpy(b->d_inst, b->h_inst.data(), sizeof(BInst) * b->n, cudaMemcpyHostToDevice));
+    if (const int rc = upload(b, b->d_inst, b->h_inst.data(), sizeof(BInst) * b->n)) return rc;
     b->tz = tile_z;
     b->stages = stages;
     b->auto_plan = false;
