@@ -58,7 +58,8 @@ cudaError_t guarded_malloc(void** p, size_t bytes)
     char* base = nullptr;
     cudaError_t e = cudaMalloc(&base, bytes + 2 * g);
     if (e != cudaSuccess) return e;
-    if ((e = cudaMemset(base, 0xFF, bytes + 2 * g)) != cudaSuccess) {
+    // (asynchronous, on the legacy stream: done before the buffer is used on another one)
+    if ((e = cudaMemset(base, 0xFF, bytes + 2 * g)) != cudaSuccess || (e = cudaStreamSynchronize(nullptr)) != cudaSuccess) {
         cudaFree(base);
         return e;
     }

@@ -2559,7 +2559,9 @@ int gs_surr_create(gs_surr** out)
     if (e == cudaSuccess) e = guarded_malloc((void**)&s->wt0x, (size_t)9 * kCinP[0] * 32 * sizeof(bf16));
     if (e == cudaSuccess) e = guarded_malloc((void**)&s->wdt5x, (size_t)9 * 16 * 32 * sizeof(bf16));
     if (e != cudaSuccess || (e = cudaMemset(s->params, 0, off * 4)) != cudaSuccess ||
-        (e = cudaMemset(s->m, 0, off * 4)) != cudaSuccess || (e = cudaMemset(s->v, 0, off * 4)) != cudaSuccess) {
+        (e = cudaMemset(s->m, 0, off * 4)) != cudaSuccess || (e = cudaMemset(s->v, 0, off * 4)) != cudaSuccess ||
+        // (asynchronous, on the legacy stream: a later gs_surr_set_stream may name one that does not wait for it)
+        (e = cudaStreamSynchronize(nullptr)) != cudaSuccess) {
         int rc = cuda_fail(e, "surrogate allocation");
         gs_surr_destroy(s);
         return rc;

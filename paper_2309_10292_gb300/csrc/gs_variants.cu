@@ -351,6 +351,8 @@ int gs_single_create(int L, double D, double dt, int dtype, int boundary, gs_sin
     if (e == cudaSuccess) e = cudaMalloc((void**)&s->d_err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(s->d_err, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(s->buf[0], 0, bytes);
+    // (asynchronous, on the legacy stream: a later gs_single_set_stream may name one that does not wait for it)
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) {
         cudaFree(s->buf[0]);
         cudaFree(s->buf[1]);
