@@ -519,10 +519,9 @@ GS_D void zmarch_body(const ZMaps& maps, const ZArgs<T>& a)
                 }
             }
         }
-        finish();
-        return;
     drain:
-        // let every copy this thread issued land before the CTA can exit
+        // let every copy this thread issued land before the CTA can exit: the
+        // consumers may have given up on one, before or after its last issue
         // (fixed 2 s budget: copies in flight always complete within it)
         for (uint32_t q = (seq > (uint32_t)S ? seq - S : 0); q < seq; ++q)
             gs_mbar_wait(&full[q % S], (q / S) & 1, 2000000000ull);

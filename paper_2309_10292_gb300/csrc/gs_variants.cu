@@ -178,8 +178,9 @@ __global__ void gs_zmarch1_kernel(const __grid_constant__ ZMaps maps, const Z1Ar
                 zp = zp + 1 == L ? 0 : zp + 1;
             }
         }
-        return;
     drain:
+        // let every copy this thread issued land before the CTA can exit: the
+        // consumers may have given up on one, before or after its last issue
         for (uint32_t q = (seq > (uint32_t)S ? seq - S : 0); q < seq; ++q)
             gs_mbar_wait(&full[q % S], (q / S) & 1, 2000000000ull);
         return;

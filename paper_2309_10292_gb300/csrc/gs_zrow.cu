@@ -168,11 +168,11 @@ __global__ void __maxnreg__(72) gs_zrow_kernel(const ZRowArgs a)
                     zp = zp + 1 == L ? 0 : zp + 1;
             }
         }
-        // after a failure: let every copy this thread issued land before the
-        // CTA can exit (fixed 2 s budget: copies in flight always complete)
-        if (!ok)
-            for (uint32_t q = (seq > (uint32_t)S ? seq - S : 0); q < seq; ++q)
-                gs_mbar_wait(&full[q % S], (q / S) & 1, 2000000000ull);
+        // let every copy this thread issued land before the CTA can exit: the
+        // consumers may have given up on one, before or after its last issue
+        // (fixed 2 s budget: copies in flight always complete)
+        for (uint32_t q = (seq > (uint32_t)S ? seq - S : 0); q < seq; ++q)
+            gs_mbar_wait(&full[q % S], (q / S) & 1, 2000000000ull);
         // the last CTA to finish zeroes the counter for the next launch
         __threadfence();
         if (atomicAdd(&a.tickets[1], 1u) == gridDim.x - 1) {
