@@ -144,7 +144,9 @@ int gs_init(gs_sim* sim);
  * than one step; its grid barrier is bounded by gs_set_fault's timeout), and
  * larger FP32 grids whose edge is no multiple of 4 a z-march on whole rows;
  * gs_get_plan then reports the z-march or plain kernel that GS_KERNEL_ZMARCH
- * or GS_KERNEL_NAIVE would mean.  FP64 fields in GS_ARITH_DS, _FX
+ * or GS_KERNEL_NAIVE would mean.  A call of one step leaves the state it starts
+ * from as it is, in the other buffer set (periodic GS_ARITH_DS, _FX and _FXF: the
+ * many-steps launch takes it for even edges up to 80).  FP64 fields in GS_ARITH_DS, _FX
  * or _FXF (periodic grids) stay in that arithmetic's packed form between the
  * steps of one call and are FP64 again when it ends, so n steps in one call
  * and in several calls can differ at the level of the FP64 rounding

@@ -190,13 +190,14 @@ static ZPlan default_tile(const gs_sim* s)
         pl.ty = (1536 + even_x / 2) / even_x;
         pl.tz = 32;
         pl.stages = 6;
-    } else if (s->dtype == GS_F64 && s->p.arith != GS_ARITH_IEEE && s->boundary == GS_BOUNDARY_HELD && L > 80 && L <= 140) {
-        // (converting every step) too few cells for the tile below: 96^3 70 -> 27
-        // us a step, 128^3 76 -> 52 (fixed point with a remainder)
+    } else if (s->dtype == GS_F64 && s->p.arith != GS_ARITH_IEEE && L > 80 && L <= 140) {
+        // (converting every step: held, or a call of one step) too few cells for
+        // the tile below: 96^3 70 -> 27 us a step, 128^3 76 -> 52 (fixed point
+        // with a remainder)
         pl.tx = even_x;
         pl.ty = pl.tz = 8;
         pl.stages = 4;
-    } else if (s->dtype == GS_F64 && s->p.arith != GS_ARITH_IEEE && L > (s->boundary == GS_BOUNDARY_HELD ? 140 : 160)) {
+    } else if (s->dtype == GS_F64 && s->p.arith != GS_ARITH_IEEE && L > 140) {
         // one CTA of up to 24 consumer warps per SM (72-80 registers a thread);
         // z-chunks as long as every SM still gets a tile.  64 x 8 x 32 with 4
         // stages -> this rule, fixed point with a remainder: 192^3 60 -> 51,
@@ -395,7 +396,7 @@ int gs_step(gs_sim* s, int64_t n)
     if (!s) return fail(GS_EINVAL, "sim is NULL");
     if (n < 0) return fail(GS_EINVAL, "n=%lld must be >= 0", (long long)n);
     int64_t i = 0;
-    if (runs_resident(s)) {
+    if (runs_resident(s) && resident_takes(s->L, s->p.arith, s->boundary == GS_BOUNDARY_HELD, n)) {
         // launches of at most kResidentSteps steps, so that no kernel runs for long
         for (; i < n;) {
             const int m = (int)std::min<int64_t>(n - i, kResidentSteps);

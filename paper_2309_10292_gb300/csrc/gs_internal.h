@@ -104,11 +104,13 @@ int launch_zrow(int L, const void* u, const void* v, void* un, void* vn, const P
 // Many steps of a small grid in one launch (gs_resident.cu): n steps from the
 // state in (u[0], v[0]), stepping between the two sets; the result is in set
 // n & 1.  bar: two zeroed words of device memory the launch leaves zeroed.
-// p.arith other than IEEE and periodic: packs (u[0], v[0]) in place.
+// p.arith other than IEEE and periodic: packs (u[0], v[0]) in place, unless the
+// call is one step (p.io == 0).
 // Returns kResidentTooLarge (nothing launched) where its CTAs cannot all be
 // resident; the caller takes the other kernels then.
 constexpr int kResidentTooLarge = 1;
 bool resident_supported(int dtype, int L, int arith, bool held);
+bool resident_takes(int L, int arith, bool held, int64_t n);  // a call of n steps, where supported
 // footprint (both buffer sets) up to which a resident step's loads are L2 hits throughout
 constexpr long long kResL2Fit = 96ll << 20;
 int launch_resident(int dtype, int L, void* const u[2], void* const v[2], int n, const Params& p, bool held, int64_t t,

@@ -125,11 +125,12 @@ GS_D void res_cell(const ResCoef<double, AR>& c, int32_t rn, double cu, double c
 
 // One step of the V cells at (x, y, z).  u, v, un, vn without __restrict__: other
 // CTAs write in one step what this one reads in the next.  AR > 0 (FP64): the
-// inputs are packed values, the outputs too unless `unpack`; with HELD, whose
-// outer layer has to keep its FP64 values to the bit, both are FP64 values and
-// every load is converted.  Returns the range word of AR = 3 (fxf_range_bad;
-// all ones: an input out of range).
-template <typename T, int V, bool NOISE, bool HELD, int AR>
+// inputs are packed values, the outputs too unless `unpack`; with CONV both are
+// FP64 values and every load is converted (HELD, whose outer layer has to keep
+// its values to the bit, and a call of one step, which leaves its input as it
+// is).  Returns the range word of AR = 3 (fxf_range_bad; all ones: an input out
+// of range).
+template <typename T, int V, bool NOISE, bool HELD, int AR, bool CONV>
 GS_D uint32_t res_group(int L, int x, int y, int z, const T* u, const T* v, T* un, T* vn, const ResCoef<T, AR>& c,
                         GsKeys k, uint32_t kk2, bool unpack)
 {
@@ -154,7 +155,7 @@ GS_D uint32_t res_group(int L, int x, int y, int z, const T* u, const T* v, T* u
     res_load<T, V>(v + izp, nv);
     T xlu = u[ixl], xru = u[ixr], xlv = v[ixl], xrv = v[ixr];
     [[maybe_unused]] T fu[V], fv[V];  // the FP64 values behind cu, cv
-    if constexpr (AR > 0 && HELD) {
+    if constexpr (CONV) {
 #pragma unroll
         for (int e = 0; e < V; ++e) {
             fu[e] = cu[e];
@@ -181,7 +182,7 @@ GS_D uint32_t res_group(int L, int x, int y, int z, const T* u, const T* v, T* u
                 gs_update_group_fxf<NOISE, true, 0>(c, pre, kk2, cu, cv, pu, pv, nu, nv, ymu, ypu, ymv, ypv, xlu, xru,
                                                     xlv, xrv, ou, ov, rng);
         }
-        if (HELD || unpack) {
+        if (CONV || unpack) {
             res_unpack<V, AR>(ou);
             res_unpack<V, AR>(ov);
         }
@@ -230,7 +231,7 @@ GS_D uint32_t res_group(int L, int x, int y, int z, const T* u, const T* v, T* u
 }
 
 // One step of all cells of a run.
-template <typename T, int V, bool NOISE, bool HELD, int AR = 0>
+template <typename T, int V, bool NOISE, bool HELD, int AR = 0, bool CONV = false>
 GS_D uint32_t res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const T* v, T* un, T* vn,
                        const ResCoef<T, AR>& c, GsKeys k, int tid, bool unpack = false)
 {
@@ -239,7 +240,7 @@ GS_D uint32_t res_rows(const ResRows& r, const ResWalk<V>& w, const T* u, const 
     const uint32_t kk2 = gs_kk2(k);
     int xv = w.xv0, y = w.y0, z = w.z0;
     for (int g = tid; g < ng; g += blockDim.x) {
-        rng |= res_group<T, V, NOISE, HELD, AR>(L, xv * V, y, z, u, v, un, vn, c, k, kk2, unpack);
+        rng |= res_group<T, V, NOISE, HELD, AR, CONV>(L, xv * V, y, z, u, v, un, vn, c, k, kk2, unpack);
         xv += w.dxv;
         y += w.dy;
         z += w.dz;
@@ -314,7 +315,7 @@ GS_D void res_shell_row(const ResShell& q, int r, int& y, int& z)
 }
 
 // One step of the walk's groups (g: the next row and group of the row) up to row re.
-template <typename T, int V, bool NOISE, bool HELD, int AR>
+template <typename T, int V, bool NOISE, bool HELD, int AR, bool CONV>
 GS_D uint32_t res_shell_rows(const ResShell& q, int2& g, int re, const T* u, const T* v, T* un, T* vn,
                              const ResCoef<T, AR>& c, GsKeys k, bool unpack)
 {
@@ -324,7 +325,7 @@ GS_D uint32_t res_shell_rows(const ResShell& q, int2& g, int re, const T* u, con
     while (g.x < re) {
         int y, z;
         res_shell_row(q, g.x, y, z);
-        rng |= res_group<T, V, NOISE, HELD, AR>(q.L, g.y * V, y, z, u, v, un, vn, c, k, kk2, unpack);
+        rng |= res_group<T, V, NOISE, HELD, AR, CONV>(q.L, g.y * V, y, z, u, v, un, vn, c, k, kk2, unpack);
         g.x += dr;
         g.y += dxv;
         if (g.y >= nxv) { g.y -= nxv; ++g.x; }
