@@ -209,8 +209,9 @@ int gs_set_plan_full(gs_sim* sim, const gs_plan* plan);
 int gs_get_plan_full(gs_sim* sim, gs_plan* out);
 
 /* Autotuner: time every candidate plan valid for this grid — the plain
- * kernel; the many-steps launch of gs_step (reported, set and cached as
- * GS_KERNEL_AUTO, when it applies); z-march tiles x z-chunks x ring depths; for FP32, temporal
+ * kernel; the default plan (reported, set and cached as GS_KERNEL_AUTO where it
+ * means gs_step's many-steps or whole-row launch, else as its z-march tile);
+ * z-march tiles x z-chunks x ring depths; for FP32, temporal
  * blocking at depths 2-8 with several tiles — over `steps_per_trial` steps
  * each (rounded up to a multiple of 12, then to whole passes of the plan's
  * depth; CUDA events on the object's stream, after warm-up launches), keep the

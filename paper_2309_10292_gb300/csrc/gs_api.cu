@@ -2,8 +2,10 @@
 // handling and error reporting around the stencil kernels (include/gs.h).
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
+#include <iterator>
 #include <map>
 #include <mutex>
 #include <vector>
@@ -657,22 +659,39 @@ static gs_plan current_plan(gs_sim* s)
     return p;
 }
 
+// z-march plans that the tuner tries for every grid, besides the default one
+// (an even cut of the row, mostly none of these: 320^3 in FP32 takes 86 us a step
+// with 160 x 10 and 103 us with the best listed tile)
+static const int kTunerTiles[][2] = {{128, 8}, {256, 4}, {64, 16}, {128, 4}, {64, 8}, {256, 8}, {128, 16}, {32, 16}, {128, 10},
+                                     {128, 12}, {256, 6}};
+static const int kTunerChunks[] = {32, 64, 128};
+static const int kTunerStages[] = {4, 6, 8};
+
+static bool tuner_lists(const ZPlan& d)
+{
+    auto has = [](const auto& a, int x) { return std::find(std::begin(a), std::end(a), x) != std::end(a); };
+    bool tile = false;
+    for (auto& t : kTunerTiles) tile |= t[0] == d.tx && t[1] == d.ty;
+    return tile && has(kTunerChunks, d.tz) && has(kTunerStages, d.stages);
+}
+
 int gs_autotune(gs_sim* s, int steps_per_trial, gs_plan* results, int max_results, int* n_results, gs_plan* best)
 {
     if (!s) return fail(GS_EINVAL, "sim is NULL");
     if (steps_per_trial < 1) return fail(GS_EINVAL, "steps_per_trial must be >= 1");
     if (max_results < 0 || (max_results > 0 && !results)) return fail(GS_EINVAL, "bad results buffer");
     const int n = (steps_per_trial + 11) / 12 * 12;
-    // candidate plans
+    // candidate plans: the plain kernel, the default plan (as such where it is
+    // more than a z-march tile), the tuner's own tiles
     std::vector<gs_plan> cand;
     cand.push_back(gs_plan{GS_KERNEL_NAIVE, 0, 0, 0, 1, 0, 0.0});
-    // the default plan where it is more than its z-march tile (also tried below)
-    if (auto_is_resident(s) || auto_is_zrow(s)) cand.push_back(gs_plan{GS_KERNEL_AUTO, 0, 0, 0, 1, 0, 0.0});
-    const int zt[][2] = {{128, 8}, {256, 4}, {64, 16}, {128, 4}, {64, 8}, {256, 8}, {128, 16}, {32, 16}, {128, 10},
-                         {128, 12}, {256, 6}};
-    for (auto& t : zt)
-        for (int tz : {32, 64, 128})
-            for (int st : {4, 6, 8}) cand.push_back(gs_plan{GS_KERNEL_ZMARCH, t[0], t[1], tz, 1, st, 0.0});
+    if (auto_is_resident(s) || auto_is_zrow(s))
+        cand.push_back(gs_plan{GS_KERNEL_AUTO, 0, 0, 0, 1, 0, 0.0});
+    else if (const ZPlan d = default_tile(s); zmarch_supported(s->dtype, s->L) && !tuner_lists(d))
+        cand.push_back(gs_plan{GS_KERNEL_ZMARCH, d.tx, d.ty, d.tz, 1, d.stages, 0.0});
+    for (auto& t : kTunerTiles)
+        for (int tz : kTunerChunks)
+            for (int st : kTunerStages) cand.push_back(gs_plan{GS_KERNEL_ZMARCH, t[0], t[1], tz, 1, st, 0.0});
     const int bt[][2] = {{64, 16}, {128, 8}, {64, 8}, {32, 16}, {128, 4}, {32, 32}};
     for (int d = 2; d <= 4; ++d)
         for (auto& t : bt)
