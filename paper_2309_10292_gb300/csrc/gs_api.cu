@@ -776,8 +776,11 @@ int gs_autotune(gs_sim* s, int steps_per_trial, gs_plan* results, int max_result
 
 // Plan cache: one text line per tuned configuration,
 //   gs-plan-v1 <key> <kernel> <tile_x> <tile_y> <tile_z> <depth> <stages> <us_per_step>
-// with key = <device name>/sm<major><minor>/L<L>/<f32|f64>/<ieee|ds>/<periodic|held>/<noise|still>
-// (spaces and '/' in the device name written as '_').
+// with key = <device name>/sm<major><minor>/L<L>/<f32|f64>/<ieee|ds|fx|fxf>/<periodic|held>/<noise|still>
+// (spaces and '/' in the device name written as '_'), then the default plan where
+// it is none of the tuner's listed ones: /auto or /<tile>.  A line from a tuner
+// that did not have it among its candidates is thus no hit (its z-march plan
+// takes 33 us a step at 128^3 in FP32, the default one 5.4).
 static int plan_key(gs_sim* s, char* key, size_t n)
 {
     int dev = 0;
@@ -788,10 +791,16 @@ static int plan_key(gs_sim* s, char* key, size_t n)
     size_t i = 0;
     for (; i < sizeof(pr.name) && pr.name[i]; ++i) name[i] = (pr.name[i] == ' ' || pr.name[i] == '/') ? '_' : pr.name[i];
     name[i] = 0;
-    snprintf(key, n, "%s/sm%d%d/L%d/%s/%s/%s/%s", name, pr.major, pr.minor, s->L, s->dtype == GS_F32 ? "f32" : "f64",
+    const ZPlan d = default_tile(s);
+    char plan[64] = "";
+    if (auto_is_resident(s) || auto_is_zrow(s))
+        snprintf(plan, sizeof plan, "/auto");
+    else if (zmarch_supported(s->dtype, s->L) && !tuner_lists(d))
+        snprintf(plan, sizeof plan, "/%dx%dx%dx%d", d.tx, d.ty, d.tz, d.stages);
+    snprintf(key, n, "%s/sm%d%d/L%d/%s/%s/%s/%s%s", name, pr.major, pr.minor, s->L, s->dtype == GS_F32 ? "f32" : "f64",
              s->p.arith == GS_ARITH_DS ? "ds" : s->p.arith == GS_ARITH_FX ? "fx" : s->p.arith == GS_ARITH_FXF ? "fxf" : "ieee",
              s->boundary == GS_BOUNDARY_HELD ? "held" : "periodic",
-             s->p.noise != 0.0 ? "noise" : "still");
+             s->p.noise != 0.0 ? "noise" : "still", plan);
     return GS_OK;
 }
 
