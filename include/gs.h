@@ -363,9 +363,9 @@ int gs_batch_set_fault(gs_batch* b, int mode, uint64_t timeout_ns);
 /* Work decomposition of the persistent kernel: z-chunk per work item
  * (1..256, default 32, or 16 for a batch of fewer than two 32-plane items per
  * CTA) and TMA ring depth (3..8, default 8).  Synchronous; drops the captured
- * graphs.  Until this call, gs_batch_set_depth or a tuned plan, a batch whose
- * arena about fits L2 (up to 140 MB in FP32, 256 MB in FP64) runs a kernel
- * without marched items: every CTA advances an equal share of all rows. */
+ * graphs.  A batch whose arena about fits L2 (up to 140 MB in FP32, 256 MB in
+ * FP64) means by 32 and 8, as from creation on, a kernel without marched items
+ * at depth 1: every CTA advances an equal share of all rows. */
 int gs_batch_set_plan(gs_batch* b, int tile_z, int stages);
 
 /* Temporal-blocking depth of the batched launch (not in the paper): D = 1
@@ -388,9 +388,9 @@ int gs_batch_set_depth(gs_batch* b, int depth);
  * one untimed run of the same length that captures the graph; CUDA events
  * on the batch's stream.  Restores every instance's fields and the step
  * counter exactly (the arena is copied to a temporary device buffer for the
- * duration) and keeps the fastest plan (where the default one of a small
- * batch wins, see gs_batch_set_plan, it stays in force, reported as z-chunk
- * 32, ring depth 8, depth 1).  *best_tile_z, *best_stages, *best_us
+ * duration) and keeps the fastest plan (gs_batch_set_plan and
+ * gs_batch_set_depth with the reported numbers set the same one on another
+ * batch of these grids).  *best_tile_z, *best_stages, *best_us
  * and *best_depth (each may be NULL) receive it and its time per step.
  * GS_EINVAL for a NULL batch or steps_per_trial < 1.  Synchronous. */
 int gs_batch_autotune(gs_batch* b, int steps_per_trial, int* best_tile_z, int* best_stages, double* best_us,

@@ -669,6 +669,8 @@ __global__ void __launch_bounds__(kBtbThreads, 1) gs_batch_tb_kernel(const __gri
 
 using namespace gs;
 
+static constexpr int kDefaultTz = 32, kDefaultStages = 8;
+
 struct gs_batch {
     int n = 0, dtype = GS_F32;
     double Du = 0, Dv = 0, dt = 0, noise = 0;
@@ -686,7 +688,7 @@ struct gs_batch {
     BCtrl* d_ctrl = nullptr;
     std::vector<ZPlan> zplan;               // per-instance plan of the sequential path
     std::vector<ZMaps> zmaps[2];            // per-instance tensor maps of the sequential path
-    int nitems = 0, tz = 32, stages = 8, main_elems = 0, row_elems = 0, field_elems = 0;
+    int nitems = 0, tz = kDefaultTz, stages = kDefaultStages, main_elems = 0, row_elems = 0, field_elems = 0;
     size_t arena_bytes = 0;
     int grid = 0;
     int64_t t = 0;
@@ -706,7 +708,8 @@ struct gs_batch {
     std::vector<int4> tb_base_items;
     int4* d_tb_items = nullptr;
     int tb_items_cap = 0, tb_nitems = 0, tb_items_grid = -1, tb_pe = 0, tb_grid = 0;
-    // small batches under the default plan run the L2-resident kernel
+    // small batches run the L2-resident kernel at depth 1 under the default
+    // plan: the one of creation, or named by its z-chunk and ring depth
     bool auto_plan = true;
     int4* d_res_tab = nullptr;  // its table (null: it does not apply)
     int res_grid = 0, res_segs = 0, res_groups = 0;
@@ -1176,7 +1179,7 @@ int gs_batch_create(int n, const int* L, const double* F, const double* k, doubl
     // (64 grids of 64^3: 58 against 51 us a step; 100 of them: 76.0 against 75.7)
     long long items32 = 0;
     for (int i = 0; i < n; ++i) items32 += (long long)run_tiles(L[i], tile_cells) * ((L[i] + 31) / 32);
-    b->tz = items32 < 4ll * num_sms() ? 16 : 32;
+    b->tz = items32 < 4ll * num_sms() ? 16 : kDefaultTz;
     // instance table, arena offsets, work items
     int nit = 0;
     long long off = 0;
@@ -1363,7 +1366,6 @@ int gs_batch_autotune(gs_batch* b, int steps_per_trial, int* best_tile_z, int* b
         rc = cuda_fail(e, "batch autotune save");
     int win_tz = tz0, win_st = st0, win_d = d0;
     double win_us = -1.0;
-    bool win_auto = false;
     auto time_plan = [&](double& us) -> int {
         int r = gs_batch_step(b, trial);  // captures the graph, warms up
         if (!r) r = gs_batch_sync(b);
@@ -1376,18 +1378,6 @@ int gs_batch_autotune(gs_batch* b, int steps_per_trial, int* best_tile_z, int* b
         us = 1e3 * ms / trial;
         return r;
     };
-    if (!rc && auto_is_resident(b)) {
-        // the default plan where it is more than its z-chunk and ring (also tried below)
-        rc = gs_batch_set_depth(b, 1);
-        if (!rc) {
-            b->auto_plan = true;
-            rc = time_plan(win_us);
-        }
-        win_auto = !rc;
-        win_tz = 32;
-        win_st = 8;
-        win_d = 1;
-    }
     for (int depth = 1; depth <= kBtbMaxDepth && !rc; ++depth) {
         if (depth > 1 && b->dtype != GS_F32) break;
         for (int tz : {16, 32, 64, 128}) {
@@ -1404,7 +1394,6 @@ int gs_batch_autotune(gs_batch* b, int steps_per_trial, int* best_tile_z, int* b
                     win_tz = tz;
                     win_st = depth > 1 ? st0 : st;
                     win_d = depth;
-                    win_auto = false;
                 }
             }
         }
@@ -1422,11 +1411,10 @@ int gs_batch_autotune(gs_batch* b, int steps_per_trial, int* best_tile_z, int* b
     b->ctrl_dirty = true;
     int rc2 = rc ? gs_batch_set_plan(b, tz0, st0) : gs_batch_set_plan(b, win_tz, win_st);
     if (!rc2) rc2 = gs_batch_set_depth(b, rc ? d0 : win_d);
-    if (!rc2 && (rc ? auto0 : win_auto)) {
-        b->auto_plan = true;
-        drop_graphs(b);
+    if (rc) {
+        b->auto_plan = auto0;
+        return rc;
     }
-    if (rc) return rc;
     if (rc2) return rc2;
     if (best_tile_z) *best_tile_z = win_tz;
     if (best_stages) *best_stages = win_st;
@@ -1532,7 +1520,7 @@ int gs_batch_set_plan(gs_batch* b, int tile_z, int stages)
     if (const int rc = upload(b, b->d_inst, b->h_inst.data(), sizeof(BInst) * b->n)) return rc;
     b->tz = tile_z;
     b->stages = stages;
-    b->auto_plan = false;
+    b->auto_plan = tile_z == kDefaultTz && stages == kDefaultStages;
     drop_graphs(b);
     if (b->depth > 1) return build_tb_tables(b, b->depth);  // the blocked items follow the z-chunk
     return GS_OK;
@@ -1548,7 +1536,6 @@ int gs_batch_set_depth(gs_batch* b, int depth)
         if (rc) return rc;
     }
     b->depth = depth;
-    b->auto_plan = false;
     drop_graphs(b);
     return GS_OK;
 }
@@ -1573,7 +1560,7 @@ int gs_batch_info(gs_batch* b, int* grid, int* items, int* cooperative, int64_t*
 {
     if (!b) return fail(GS_EINVAL, "batch is NULL");
     if (depth) *depth = b->depth;
-    const bool res = runs_resident(b) && b->d_res_tab;
+    const bool res = runs_resident(b);
     if (grid) *grid = res ? b->res_grid : b->depth > 1 ? b->tb_grid : b->grid;
     if (items) *items = res ? b->res_segs : b->depth > 1 ? b->tb_nitems : b->nitems;
     if (cooperative) *cooperative = b->cooperative ? 1 : 0;
