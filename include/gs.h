@@ -140,7 +140,7 @@ int gs_init(gs_sim* sim);
  * (GS_KERNEL_AUTO) grids of up to 256^3 cells (FP32 edges that are no multiple
  * of 4: 218^3, or 202^3 with an odd edge; GS_ARITH_DS, _FX and _FXF: 160^3, or
  * 180^3 with an odd edge, and 80^3 / 120^3 with the held boundary) run up to 4096
- * steps in one launch (a cooperative one when it holds more
+ * steps, and some 60 ms, in one launch (a cooperative one when it holds more
  * than one step; its grid barrier is bounded by gs_set_fault's timeout), and
  * larger FP32 grids whose edge is no multiple of 4 a z-march on whole rows;
  * gs_get_plan then reports the z-march or plain kernel that GS_KERNEL_ZMARCH

@@ -236,8 +236,6 @@ static int default_plan(gs_sim* s)
     return GS_OK;
 }
 
-static constexpr int kResidentSteps = 4096;
-
 // whether the default plan means the resident kernel (the injected fault is
 // one of the TMA producer)
 static bool auto_is_resident(const gs_sim* s)
@@ -399,9 +397,9 @@ int gs_step(gs_sim* s, int64_t n)
     if (n < 0) return fail(GS_EINVAL, "n=%lld must be >= 0", (long long)n);
     int64_t i = 0;
     if (runs_resident(s) && resident_takes(s->L, s->p.arith, s->boundary == GS_BOUNDARY_HELD, n)) {
-        // launches of at most kResidentSteps steps, so that no kernel runs for long
+        const int64_t longest = resident_max_steps(s->dtype, s->L);
         for (; i < n;) {
-            const int m = (int)std::min<int64_t>(n - i, kResidentSteps);
+            const int m = (int)std::min(n - i, longest);
             const int in = s->cur, outs = 1 - s->cur;
             void* const u[2] = {s->buf[in][0], s->buf[outs][0]};
             void* const v[2] = {s->buf[in][1], s->buf[outs][1]};

@@ -110,6 +110,7 @@ int launch_zrow(int L, const void* u, const void* v, void* un, void* vn, const P
 // resident; the caller takes the other kernels then.
 constexpr int kResidentTooLarge = 1;
 bool resident_supported(int dtype, int L, int arith, bool held);
+int resident_max_steps(int dtype, int L);  // steps that one launch may hold
 bool resident_takes(int L, int arith, bool held, int64_t n);  // a call of n steps, where supported
 // footprint (both buffer sets) up to which a resident step's loads are L2 hits throughout
 constexpr long long kResL2Fit = 96ll << 20;

@@ -239,6 +239,15 @@ bool resident_supported(int dtype, int L, int arith, bool held)
     return L <= 256;
 }
 
+// A launch holds every SM until it ends, and work on other streams waits: about
+// 60 ms at most (5 ps per cell and step in FP32, 201^3; 42 in IEEE FP64 and up to
+// 60 in the other arithmetics with the held layer, 72^3), and 4096 steps.
+int resident_max_steps(int dtype, int L)
+{
+    const long long cell_steps = dtype == GS_F32 ? 10'000'000'000ll : 1'200'000'000ll;
+    return (int)std::min<long long>(4096, std::max<long long>(2, cell_steps / ((long long)L * L * L)));
+}
+
 // Calls that the kernel takes.  Periodic FP64 fields in another arithmetic than
 // IEEE are packed in place, which a call of two or more steps may do (its second
 // step overwrites the input anyway).  A call of one step leaves its input as it
