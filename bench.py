@@ -630,6 +630,25 @@ def bench_surrogate(args, stream):
             "fp32_stencil_vs_fp64_stencil": err((up, vp), (u64, v64))}
 
 
+def launch_summary(plan, L, steps, launches):
+    """Kernel name, steps per launch, what bounds it and the bytes of its steps
+    (u and v read and written once per step, or per pass of a blocked plan) for
+    `steps` stencil steps of an L^3 FP32 grid in `launches` launches.  A plan
+    reported as GS_KERNEL_AUTO is the many-steps launch, whose fields stay in
+    L2, or (one step per launch) the z-march on whole rows."""
+    from paper_2309_10292_gb300 import gs
+    step_bytes = 16.0 * L ** 3
+    if plan["kernel"] == gs.GS_KERNEL_AUTO:
+        per = steps / launches
+        if per > 1:
+            return "gs_resident_kernel<float, noise>", per, "issue (fields in L2)", step_bytes * per
+        return "gs_zrow_kernel<noise>", per, "issue", step_bytes
+    if plan["kernel"] == gs.GS_KERNEL_TBLOCK:
+        return f"gs_tblock_kernel<noise, {plan['depth']}>", plan["depth"], "hbm", step_bytes
+    name = "gs_naive_kernel" if plan["kernel"] == gs.GS_KERNEL_NAIVE else "gs_zmarch_kernel"
+    return name + "<float, noise>", 1, "hbm", step_bytes
+
+
 def run_ours(args):
     import numpy as np
     import torch
@@ -695,10 +714,8 @@ def run_ours(args):
     value = whole_job_rate(ws, cells * args.time_steps * args.steps, total_ms / 1e3) / 1e9
     per_launch_s = step_ms / 1e3 / stencil_launches
     hbm_peak, peak_kind = load_peaks()
-    alg_bytes = 16.0 * cells  # one read and one write of u and v per pass
+    kname, steps_per_launch, bound, alg_bytes = launch_summary(plan, L, args.time_steps * args.steps, stencil_launches)
     achieved = alg_bytes / per_launch_s / 1e9
-    kname = {gs.GS_KERNEL_NAIVE: "gs_naive_kernel<float, noise>", gs.GS_KERNEL_ZMARCH: "gs_zmarch_kernel<float, noise>",
-             gs.GS_KERNEL_TBLOCK: f"gs_tblock_kernel<noise, {plan['depth']}>"}[plan["kernel"]]
     traffic = profiled_traffic() if plan["kernel"] == gs.GS_KERNEL_ZMARCH else None
 
     # end to end through the C-ABI with host buffers: every bench step copies
@@ -856,10 +873,10 @@ def run_ours(args):
                        "l2": "inputs larger than L2 (4 field buffers of %.2f GB)" % (cells * 4 / 1e9),
                        "parallelism": "replicas" if ws > 1 else "single GPU",
                        "source_sha256_16": source_digest()},
-            "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
+            "roofline": {"bound": bound, "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                          "frac": achieved / hbm_peak, "traffic": traffic,
                          "kernel": kname, "launches": stencil_launches,
-                         "steps_per_launch": plan["depth"] if plan["kernel"] == gs.GS_KERNEL_TBLOCK else 1,
+                         "steps_per_launch": steps_per_launch,
                          "peak_kind": f"{peak_kind} (MEASURED_PEAKS.json hbm_gbs)" if peak_kind == "measured"
                          else "fallback 6.8 TB/s",
                          "algorithmic_bytes_per_launch": alg_bytes,
