@@ -92,7 +92,14 @@ struct GsCoefFXF {
     int32_t KF;    // F dt in sixteenths of a unit, rounded ...
     float rF;      // ... and the rest
     int dt_one;    // dt == 1: the product (v^2) dt is skipped
-    // for the two-cell form: {c1, c1}, {-c1, -c1}, {-c2, -c2} of the five
+};
+static_assert(sizeof(GsCoefFXF) == 60, "what the plain kernel takes: see below");
+
+// ... and with the operands of the two-cell form.  Apart from those above: the
+// plain kernel compiled with them among its parameters keeps 32 registers in
+// place of 40 and takes 69 in place of 65 us a step (181^3 without noise).
+struct GsCoefFXF2 : GsCoefFXF {
+    // {c1, c1}, {-c1, -c1}, {-c2, -c2} of the five
     // products above (a, b, f, k, n), {rF, rF}, and the packed constants
     // -1, 1/16, 4 2^-22, -4 2^-22 (64-bit operands from the parameter space)
     gs_f2 p1[5], m1[5], m2[5], rF2, neg, sixteenth, vs, mvs;
@@ -111,9 +118,9 @@ inline void fxf_split_host(double d, float& hi, float& lo)
     lo = (float)(d - (double)hi);
 }
 
-inline GsCoefFXF gs_make_coef_fxf(double Du, double Dv, double F, double k, double dt, double noise)
+inline GsCoefFXF2 gs_make_coef_fxf(double Du, double Dv, double F, double k, double dt, double noise)
 {
-    GsCoefFXF c;
+    GsCoefFXF2 c;
     fxf_split_host(Du / 6.0 * dt * 16.0, c.a1, c.a2);
     fxf_split_host(Dv / 6.0 * dt * 16.0, c.b1, c.b2);
     fxf_split_host((Du + F) * dt * 16.0, c.f1, c.f2);
@@ -261,7 +268,7 @@ GS_D void gs_update_fxf(const GsCoefFXF& c, GsFxf u, GsFxf v, int32_t SU, float 
 // instead of 114 scalar ones: 256 x 6 x 64 tiles, 512^3 838 -> 813 us a step with
 // noise, 764 -> 732 without; 256^3 113.5 -> 111.0 and 104.1 -> 101.1.
 template <bool NOISE>
-GS_D void gs_update_fxf2(const GsCoefFXF& c, const GsFxf (&u)[2], const GsFxf (&v)[2], const int32_t (&SU)[2],
+GS_D void gs_update_fxf2(const GsCoefFXF2& c, const GsFxf (&u)[2], const GsFxf (&v)[2], const int32_t (&SU)[2],
                          const float (&SLU)[2], const int32_t (&SV)[2], const float (&SLV)[2], const int32_t (&rnum)[2],
                          GsFxf (&un)[2], GsFxf (&vn)[2], uint32_t& rng)
 {
@@ -354,7 +361,7 @@ GS_D void gs_update_fxf2(const GsCoefFXF& c, const GsFxf (&u)[2], const GsFxf (&
 // A 2-cell group of cells whose inputs are packed pairs (fxf_pack); writes
 // packed pairs (PACK) or FP64 values.
 template <bool NOISE, bool PACK, int DT>
-GS_D void gs_update_group_fxf(const GsCoefFXF& c, uint32_t pre, uint32_t kk2, const double* cu, const double* cv,
+GS_D void gs_update_group_fxf(const GsCoefFXF2& c, uint32_t pre, uint32_t kk2, const double* cu, const double* cv,
                               const double* pu, const double* pv, const double* nu, const double* nv,
                               const double* ymu, const double* ypu, const double* ymv, const double* ypv,
                               double xlu, double xru, double xlv, double xrv, double* ou, double* ov, uint32_t& rng)

@@ -62,7 +62,7 @@ struct ResWalk {
 // fixed point with a float remainder).
 template <typename T, int AR>
 using ResCoef = std::conditional_t<AR == 0, GsCoef<T>,
-                                   std::conditional_t<AR == 1, GsCoefDS, std::conditional_t<AR == 2, GsCoefFX, GsCoefFXF>>>;
+                                   std::conditional_t<AR == 1, GsCoefDS, std::conditional_t<AR == 2, GsCoefFX, GsCoefFXF2>>>;
 
 // V cells from FP64 to AR's packed values; false: a value out of its range
 template <int V, int AR>

@@ -300,7 +300,7 @@ struct ZArgs {
     GsCoef<T> c;
     GsCoefDS cds;            // the same coefficients as double-single pairs (DS kernels)
     GsCoefFX cfx;            // and in fixed point (FX kernels)
-    GsCoefFXF cfxf;          // and as float pairs for the fixed point with a remainder (FXF kernels)
+    GsCoefFXF2 cfxf;         // and as float pairs for the fixed point with a remainder (FXF kernels)
     GsKeys keys;
     int* err;
     uint64_t timeout_ns;
