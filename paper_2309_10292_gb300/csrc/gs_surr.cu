@@ -321,10 +321,10 @@ struct WgArgs {
     float* dw;       // [27][cin][cout] (fp32, accumulated with atomics)
     int N, L, GST, cin, cout;
     int rows;        // rows of a CTA's column (divides L)
+    int planes;      // planes of a unit
 };
 
 constexpr int kWgThreads = 864;  // one warp per tap
-constexpr int kWgPlanes = 4;     // planes of a unit
 
 // Like gs_conv_kernel a CTA advances along z through columns of `rows` rows,
 // with the input planes in a ring of 4 slots and the gradient planes in a ring
@@ -358,16 +358,16 @@ __global__ void __launch_bounds__(kWgThreads, 1) gs_wgrad_kernel(const WgArgs a)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[mt][nt][i] = 0.f;
 
-    // units of kWgPlanes planes, dealt out round robin: every CTA's sums run over
+    // units of a.planes planes, dealt out round robin: every CTA's sums run over
     // a sample of the whole grid, so that the partial sums grow alike and the
     // tensor cores' truncated FP32 accumulation loses alike in all of them
     // (contiguous runs of planes: 3 % faster, but weight gradients of smooth
     // fields up to 1.2e-5 of their norm from sums dealt out this way)
-    const int nz = (L + kWgPlanes - 1) / kWgPlanes;
+    const int nz = (L + a.planes - 1) / a.planes;
     const long long units = (long long)a.N * ngrp * nseg * nz;
     for (long long unit = blockIdx.x; unit < units; unit += gridDim.x) {
         const long long col = unit / nz;
-        const int z0 = (int)(unit - col * nz) * kWgPlanes, z1 = min(L, z0 + kWgPlanes);
+        const int z0 = (int)(unit - col * nz) * a.planes, z1 = min(L, z0 + a.planes);
         const int seg = (int)(col % nseg);
         const int yg = (int)((col / nseg) % ngrp);
         const int n = (int)(col / nseg / ngrp);
@@ -2143,14 +2143,20 @@ int wgrad_launch(gs_surr* s, WgArgs a)
     auto bytes = [&](int r) { return (size_t)4 * (r + 2) * (SEG + 2) * CINP * 2 + (size_t)2 * r * SEG * NP * 2; };
     a.rows = 8;
     while (bytes(a.rows) > 227 * 1024) a.rows /= 2;
+    // units of 4 planes; fewer, and then columns of 4 rows, where they would be
+    // 19 at most (us per training step at 16^3, 4 planes of 8 rows -> this rule: one
+    // grid 377 -> 321, two 376 -> 336; from three on four planes)
+    a.planes = 4;
+    auto count = [&]() { return (long long)a.N * ((a.L + a.planes - 1) / a.planes) * (a.L / a.rows) * (a.L / SEG); };
+    while (a.planes > 1 && 8 * count() <= num_sms()) a.planes /= 2;
+    if (a.rows > 4 && 8 * count() <= num_sms()) a.rows = 4;
     const size_t smem = bytes(a.rows);
     auto k = gs_wgrad_kernel<CINP, NP>;
     GS_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     GS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kWgThreads, smem));
     if (per_sm < 1) return fail(GS_EINVAL, "weight-gradient tile does not fit on an SM");
-    const long long units = (long long)a.N * ((a.L + kWgPlanes - 1) / kWgPlanes) * (a.L / a.rows) * (a.L / SEG);
-    const int grid = (int)std::min<long long>(units, (long long)per_sm * num_sms());
+    const int grid = (int)std::min<long long>(count(), (long long)per_sm * num_sms());
     k<<<grid, kWgThreads, smem, s->stream>>>(a);
     GS_CUDA_TRY(cudaGetLastError());
     s->launches += 1;
