@@ -113,6 +113,25 @@ int num_sms()
     return n > 0 ? n : 1;
 }
 
+int usable_sms()
+{
+    const int all = num_sms();
+    void *cur = nullptr, *get = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    CUcontext ctx = nullptr;
+    CUdevResource r;
+    memset(&r, 0, sizeof r);
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &cur, 4000, cudaEnableDefault, &q) != cudaSuccess || !cur ||
+        cudaGetDriverEntryPointByVersion("cuCtxGetDevResource", &get, 12040, cudaEnableDefault, &q) != cudaSuccess || !get ||
+        reinterpret_cast<CUresult (*)(CUcontext*)>(cur)(&ctx) != CUDA_SUCCESS || !ctx ||
+        reinterpret_cast<CUresult (*)(CUcontext, CUdevResource*, CUdevResourceType)>(get)(ctx, &r, CU_DEV_RESOURCE_TYPE_SM) !=
+            CUDA_SUCCESS) {
+        cudaGetLastError();
+        return all;
+    }
+    return r.sm.smCount > 0 ? std::min(all, (int)r.sm.smCount) : all;
+}
+
 static PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 static std::once_flag g_encode_once;
 

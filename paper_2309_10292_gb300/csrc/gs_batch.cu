@@ -696,6 +696,10 @@ struct gs_batch {
     bool ctrl_dirty = true;
     cudaStream_t stream = nullptr;
     cudaStream_t cap = nullptr;
+    // SMs of the context that the graphs' launches belong to (cap's).  Grids are
+    // sized by them: the launch of a graph does not report a cooperative kernel
+    // whose CTAs cannot all be resident there, and never ends
+    int sms = 1;
     std::map<int64_t, cudaGraphExec_t> graphs;
     int64_t launches = 0;
     uint64_t timeout_ns = 2000000000ull;
@@ -899,7 +903,7 @@ static int plain_prepare(gs_batch* b, int64_t n, BArgs<T>& a, size_t& smem)
     int per_sm = 0;
     GS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBatchThreads, smem));
     if (per_sm < 1) return fail(GS_EINVAL, "batch kernel does not fit on an SM");
-    const int grid = std::min(per_sm * num_sms(), (int)b->base_items.size());
+    const int grid = std::min(per_sm * b->sms, (int)b->base_items.size());
     if (b->items_grid != grid) {
         // cut the last items for this grid (once per plan)
         std::vector<int4> items;
@@ -939,7 +943,7 @@ static int tb_prepare(gs_batch* b, int64_t npasses, BtbArgs& a, size_t& smem)
     int per_sm = 0;
     GS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBtbThreads, smem));
     if (per_sm < 1) return fail(GS_EINVAL, "blocked batch kernel does not fit on an SM");
-    const int grid = std::min(per_sm * num_sms(), (int)b->tb_base_items.size());
+    const int grid = std::min(per_sm * b->sms, (int)b->tb_base_items.size());
     if (b->tb_items_grid != grid) {
         std::vector<int4> items;
         split_last(b->tb_base_items, grid / 2, 4, false, items);  // the blocked item marches up only
@@ -1006,7 +1010,7 @@ static int plan_res_table(gs_batch* b)
     const int V = b->dtype == GS_F32 ? 4 : 2;
     long long total = 0;
     for (int L : b->L) total += (long long)L * L * (L / V);
-    const int grid = (int)std::min<long long>(num_sms(), std::max<long long>(1, total / 128));
+    const int grid = (int)std::min<long long>(b->sms, std::max<long long>(1, total / 128));
     std::vector<int4> head(grid, int4{0, 0, 0, 0}), segs;
     long long pos = 0;  // groups before the instance
     int cta = 0;
@@ -1167,6 +1171,7 @@ int gs_batch_create(int n, const int* L, const double* F, const double* k, doubl
     b->dt = dt;
     b->noise = noise;
     b->seed = seed;
+    b->sms = usable_sms();
     b->L.assign(L, L + n);
     b->F.assign(F, F + n);
     b->k.assign(k, k + n);
@@ -1179,7 +1184,7 @@ int gs_batch_create(int n, const int* L, const double* F, const double* k, doubl
     // (64 grids of 64^3: 58 against 51 us a step; 100 of them: 76.0 against 75.7)
     long long items32 = 0;
     for (int i = 0; i < n; ++i) items32 += (long long)run_tiles(L[i], tile_cells) * ((L[i] + 31) / 32);
-    b->tz = items32 < 4ll * num_sms() ? 16 : kDefaultTz;
+    b->tz = items32 < 4ll * b->sms ? 16 : kDefaultTz;
     // instance table, arena offsets, work items
     int nit = 0;
     long long off = 0;
@@ -1638,7 +1643,7 @@ static int noalloc_launch_t(char* scratch, void* arena, int n, int nitems, int m
     GS_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kBatchThreads, smem));
     if (per_sm < 1) return fail(GS_EINVAL, "batch kernel does not fit on an SM");
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(std::min(per_sm * num_sms(), nitems));
+    cfg.gridDim = dim3(std::min(per_sm * usable_sms(), nitems));
     cfg.blockDim = dim3(kBatchThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;

@@ -37,6 +37,8 @@ int cuda_fail(cudaError_t e, const char* what);
 
 int elem_size(int dtype);
 int num_sms();
+// SMs that kernels of the current context may use (a green context: its share)
+int usable_sms();
 
 // Library-owned device allocations that honour the guard-band checking aid
 // (gs_set_alloc_guard): with a guard of G bytes the buffer sits between two
