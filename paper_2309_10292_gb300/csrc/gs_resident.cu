@@ -123,12 +123,17 @@ static ResCoef<T, AR> res_coef(const Params& p)
 // Whether a brick steps its inner rows under the barrier.  us per step without
 // and with: FP32 64^3 2.26 / 2.29, 80^3 3.09 / 2.45, 96^3 3.89 / 3.32, 128^3 6.44 /
 // 5.40, 192^3 20.1 / 18.5, 256^3 48.8 / 48.9 (without noise 46.1 / 47.6, held 54.3 /
-// 49.4); fixed point with a remainder 64^3 3.76 / 3.68, 128^3 15.4 / 14.75, 160^3
-// 35.6 / 36.4.
-static bool shell_pays(int dtype_bytes, int L, bool held)
+// 49.4); fixed point with a remainder 64^3 3.84 / 3.77, 80^3 5.74 / 4.87, 128^3
+// 15.4 / 15.1, 140^3 21.7 / 21.3, 160^3 35.6 / 36.4; fixed point 64^3 5.35 / 5.37,
+// 72^3 7.12 / 6.66, 128^3 26.2 / 25.3, 140^3 36.0 / 36.0; double-single 64^3 4.61 /
+// 4.69, 72^3 6.53 / 5.98, 112^3 16.8 / 16.4, 128^3 21.0 / 21.2.  Held, converting at
+// every load: 64^3 13.0 / 13.4 (double-single), 72^3 19.6 / 21.0 (fixed point), with
+// a remainder 15.7 / 15.3, 80^3 22.0 / 21.4, 25.5 / 24.8, with a remainder 20.3 / 19.1.
+static bool shell_pays(int arith, int dtype_bytes, int L, bool held)
 {
-    if (dtype_bytes == 8) return L >= 64 && L <= 140;
-    return L >= 72 && (held || L <= 224);
+    if (dtype_bytes == 4) return L >= 72 && (held || L <= 224);
+    if (held) return L > (arith == GS_ARITH_FXF ? 64 : 72);
+    return L >= (arith == GS_ARITH_FXF ? 64 : 68) && L <= (arith == GS_ARITH_DS ? 120 : 140);
 }
 
 template <typename T, int V, bool NOISE, bool HELD, int AR, bool CONV = (AR > 0 && HELD)>
@@ -204,7 +209,7 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
             if (!wide) kern = gs_resident_kernel<T, V, NOISE, HELD, AR, CONV, false, 512>;
         }
         if constexpr (V == GsVec<T>::N && (sizeof(T) == 4 || AR > 0)) {
-            if (a.ny && n > 1 && shell_pays(sizeof(T), L, HELD))
+            if (a.ny && n > 1 && shell_pays(AR, sizeof(T), L, HELD))
                 kern = wide ? gs_resident_kernel<T, V, NOISE, HELD, AR, CONV, true, 1024>
                             : gs_resident_kernel<T, V, NOISE, HELD, AR, CONV, true, 512>;
         }
