@@ -132,6 +132,23 @@ int usable_sms()
     return r.sm.smCount > 0 ? std::min(all, (int)r.sm.smCount) : all;
 }
 
+bool captured_on_part(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();  // (the launch meets the same error)
+    if (st != cudaStreamCaptureStatusActive) return false;
+    if (usable_sms() < num_sms()) return true;
+    void* get = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    CUgreenCtx green = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuStreamGetGreenCtx", &get, 12040, cudaEnableDefault, &q) != cudaSuccess || !get ||
+        reinterpret_cast<CUresult (*)(CUstream, CUgreenCtx*)>(get)((CUstream)s, &green) != CUDA_SUCCESS) {
+        cudaGetLastError();
+        return false;
+    }
+    return green != nullptr;
+}
+
 static PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 static std::once_flag g_encode_once;
 

@@ -39,6 +39,9 @@ int elem_size(int dtype);
 int num_sms();
 // SMs that kernels of the current context may use (a green context: its share)
 int usable_sms();
+// whether s is being captured in, or belongs to, a context that may use part of
+// the SMs only (a green one)
+bool captured_on_part(cudaStream_t s);
 
 // Library-owned device allocations that honour the guard-band checking aid
 // (gs_set_alloc_guard): with a guard of G bytes the buffer sits between two

@@ -214,6 +214,9 @@ static int resident_launch_t(int L, void* const u[2], void* const v[2], int n, c
                             : gs_resident_kernel<T, V, NOISE, HELD, AR, CONV, true, 512>;
         }
     }
+    // (a graph's launch does not report a cooperative kernel that cannot be
+    // resident, and never ends)
+    if (cfg.numAttrs && captured_on_part(s)) return kResidentTooLarge;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a);
     if (e == cudaErrorCooperativeLaunchTooLarge) {
         // (a context that may use part of the SMs only)
