@@ -16,7 +16,7 @@ from __future__ import annotations
 import argparse
 import json
 
-KERNELS = {"naive": 1, "zmarch": 2, "tblock": 3}
+KERNELS = {"auto": 0, "naive": 1, "zmarch": 2, "tblock": 3}
 
 
 def main(argv=None):
@@ -28,7 +28,7 @@ def main(argv=None):
     ap.add_argument("--dtype", default="f32", choices=["f32", "f64"])
     ap.add_argument("--arith", default="ieee", choices=["ieee", "ds", "fx", "fxf"])
     ap.add_argument("--noise", type=float, default=0.1)
-    ap.add_argument("--plan", default="", help="kernel,tile_x,tile_y,tile_z[,depth[,stages]]; empty: autotune")
+    ap.add_argument("--plan", default="", help="auto (the default plan) or kernel,tile_x,tile_y,tile_z[,depth[,stages]]; empty: autotune")
     ap.add_argument("--steps", type=int, default=100, help="timed steps")
     ap.add_argument("--warmup", type=int, default=5)
     ap.add_argument("--batch", action="store_true", help="time the 256-instance batched launch")
