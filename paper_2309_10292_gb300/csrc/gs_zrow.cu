@@ -12,10 +12,10 @@
 // apart when the edge is odd (any alignment, no bank conflicts), a pair when it
 // is even (every row start is 8-byte aligned).
 //
-// Bound by instruction issue (ncu: 84 thread instructions per cell and 77 % of
-// issue slots at 414^3, 110 and 68 % at 251^3, DRAM traffic 0.98 of 16 bytes a
+// Bound by instruction issue (ncu: 79 thread instructions per cell and 77 % of
+// issue slots at 414^3, 103 and 68 % at 251^3, DRAM traffic 0.98 of 16 bytes a
 // cell).  us per step with noise, plain kernel -> this one: 222^3 84 -> 50, 250^3
-// 118 -> 60, 251^3 119 -> 68, 414^3 518 -> 201 (353 GCUPS), 501^3 914 -> 458, 777^3
+// 118 -> 59, 251^3 119 -> 68, 414^3 518 -> 199 (357 GCUPS), 501^3 914 -> 458, 777^3
 // 3393 -> 1660, 1302^3 18000 -> 6680.  With four single cells per thread a block
 // apart (y neighbours from shared memory too) 250^3 took 64, 414^3 231 us.
 #include <algorithm>
