@@ -209,6 +209,35 @@ static bool finite_params(double a, double b, double c, double d, double e, doub
            std::isfinite(e) && std::isfinite(f);
 }
 
+// z-chunk of a grid of `cols` columns whose tiles one CTA per SM takes round robin,
+// the tiles of the last, partial round cut along z (the FP64 arithmetics other
+// than IEEE).  A step takes as long as its busiest CTA, which goes through planes
+// at a constant rate: its tiles' own and two more for each.  Equal chunks of up to
+// 64 planes, or those with the fewest such planes where that is over 2 % less.  us
+// per step, noise 0.1, chunks of 64 with a rest (32, 16 on small grids) -> this
+// rule: fixed point with a remainder 162^3 41.3 -> 38.6, 200^3 77.2 -> 65.1, 258^3
+// (4 x 64 + 2 planes: 132 in place of 88 for the busiest CTA) 197 -> 134, 300^3 204
+// -> 192, 388^3 468 -> 427; double-single 258^3 306 -> 208, held 552 -> 394
+static int round_robin_chunk(int L, int cols)
+{
+    const int sms = num_sms();
+    auto planes = [&](int h) {
+        const int tiles = cols * ((L + h - 1) / h), G = std::min(sms, tiles), rem = tiles % G;
+        const int parts = rem ? G / rem : 1;
+        return tiles / G * (h + 2) + (rem ? (h + parts - 1) / parts + 2 : 0);
+    };
+    auto equal = [&](int nz) { return (L + nz - 1) / nz; };
+    int tz = equal((L + 63) / 64);
+    int best = planes(tz) * 49 / 50;
+    for (int nz = 1; 8 * nz <= L; ++nz) {
+        const int n = planes(equal(nz));
+        if (n >= best) continue;
+        best = n;
+        tz = equal(nz);
+    }
+    return tz;
+}
+
 // The z-march tile of the default plan.  The grid is cut in x into equal tiles
 // of up to 256 cells (an uneven cut idles threads: 320 = 2 x 160 runs at 86 us a
 // step in FP32, as 3 x 128 at 103 us), in y so that a tile fills its block.
@@ -236,16 +265,14 @@ static ZPlan default_tile(const gs_sim* s)
         pl.ty = pl.tz = 8;
         pl.stages = 4;
     } else if (s->dtype == GS_F64 && s->p.arith != GS_ARITH_IEEE && L > 140) {
-        // one CTA of up to 24 consumer warps per SM (72-80 registers a thread);
-        // z-chunks as long as every SM still gets a tile.  64 x 8 x 32 with 4
+        // one CTA of up to 24 consumer warps per SM (72-80 registers a thread).  64 x 8 x 32 with 4
         // stages -> this rule, fixed point with a remainder: 192^3 60 -> 51,
         // 256^3 125 -> 109, 320^3 278 -> 234, 512^3 980 -> 870 (held: 160^3 112 ->
         // 81, 256^3 352 -> 263, 354^3 983 -> 755); double-single 256^3 210 -> 165,
         // fixed point 222 -> 189
         pl.tx = even_x;
         pl.ty = 1536 / even_x;
-        const int cols = (L + pl.tx - 1) / pl.tx * ((L + pl.ty - 1) / pl.ty);
-        pl.tz = cols * ((L + 63) / 64) >= num_sms() ? 64 : cols * ((L + 31) / 32) >= num_sms() * 9 / 10 ? 32 : 16;
+        pl.tz = round_robin_chunk(L, (L + pl.tx - 1) / pl.tx * ((L + pl.ty - 1) / pl.ty));
         pl.stages = s->p.arith == GS_ARITH_FXF ? 6 : 4;
     } else {
         pl.tx = std::min(s->dtype == GS_F32 ? 128 : 64, L);
