@@ -276,11 +276,11 @@ static ZPlan default_tile(const gs_sim* s)
         pl.ty = pl.tz = 8;
         pl.stages = 4;
     } else if (s->dtype == GS_F64 && s->p.arith != GS_ARITH_IEEE && L > 140) {
-        // one CTA of up to 24 consumer warps per SM (72-80 registers a thread).  64 x 8 x 32 with 4
-        // stages -> this rule, fixed point with a remainder: 192^3 60 -> 51,
-        // 256^3 125 -> 109, 320^3 278 -> 234, 512^3 980 -> 870 (held: 160^3 112 ->
-        // 81, 256^3 352 -> 263, 354^3 983 -> 755); double-single 256^3 210 -> 165,
-        // fixed point 222 -> 189
+        // one CTA of up to 24 consumer warps per SM (72-80 registers a thread).
+        // 64 x 8 x 32 with 4 stages -> this rule, fixed point with a remainder:
+        // 192^3 60 -> 51, 256^3 125 -> 109, 320^3 278 -> 234, 512^3 980 -> 870 (held:
+        // 160^3 112 -> 80, 256^3 352 -> 262, 354^3 983 -> 713); double-single 256^3
+        // 210 -> 165, fixed point 222 -> 189
         pl.tx = even_x;
         pl.ty = 1536 / even_x;
         pl.tz = round_robin_chunk(L, (L + pl.tx - 1) / pl.tx * ((L + pl.ty - 1) / pl.ty));
